@@ -11,9 +11,7 @@
 // fixed order (per-block partials, then an ordered finishing pass), so the
 // training is bitwise repeatable.
 #include <atomic>
-#include <cuda.h>
 #include <cuda_bf16.h>
-#include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <cstdlib>
@@ -22,7 +20,6 @@
 
 #include "internal.h"
 #include "nn.h"
-#include "umma.cuh"
 
 namespace lbm {
 namespace nn {
@@ -738,42 +735,6 @@ __global__ void __launch_bounds__(256) conv1x1_small_kernel(const TI *__restrict
     }
 }
 
-// 3^3 convolution on the 5th-generation tensor cores (tcgen05.mma with the
-// accumulator in tensor memory).  A CTA of 4 warps owns a tile of 8 x 16
-// voxels of one z-plane (M = 128 GEMM rows) and CO output channels (N).  Per
-// 16 input channels it stages the x halo (10 x 18 x 3 voxels) and the
-// weights of all 27 taps in the canonical K-major core-matrix layout (8 rows
-// x 16 bytes per core matrix):
-//   halo   [kg 2][z 3][y 18][x 10] x 16 B: the 8 rows of a core matrix are 8
-//          consecutive x voxels, so tap (dz, dy, dx) is the same descriptor
-//          shifted by ((dz * 18 + dy) * 10 + dx) * 16 bytes; SBO (next 8 rows
-//          = next y row) = 160 B, LBO (next 8 channels) = 540 * 16 B;
-//   weights [tap 27][kg 2][co CO] x 16 B: SBO (next 8 channels out) = 128 B,
-//          LBO (next 8 channels in) = CO * 16 B.
-// One thread issues the 27 MMAs (K = 16 each) and commits them to an
-// mbarrier; everyone waits (bounded) before the buffers are restaged.  The
-// epilogue reads each thread's accumulator row (TMEM lane = voxel) with
-// tcgen05.ld and writes bias + activation.  A wait that runs out sets *err.
-constexpr int kUmX = 8, kUmY = 16;
-constexpr int kUmHX = kUmX + 2, kUmHY = kUmY + 2, kUmHZ = 3;
-constexpr int kUmHalo = kUmHX * kUmHY * kUmHZ;                // 540 voxels
-constexpr unsigned kUmHaloOff = 128;                         // after the barrier and TMEM slot
-constexpr unsigned kUmHaloBytes = 2u * kUmHalo * 16u;        // 17280
-template <int CO>
-constexpr unsigned um_smem_bytes()
-{
-    return kUmHaloOff + kUmHaloBytes + 27u * 2u * CO * 16u;
-}
-constexpr unsigned kUmWaitPolls = 1u << 22;  // ~0.3 s of polling before giving up
-// TMEM columns a CTA allocates (the accumulator needs CO, at least 32);
-// DMRT_UMMA_TMEM_COLS raises it (a power of two up to 512).
-#ifndef DMRT_UMMA_CTAS_PER_SM
-#define DMRT_UMMA_CTAS_PER_SM 4
-#endif
-#ifndef DMRT_UMMA_TMEM_COLS
-#define DMRT_UMMA_TMEM_COLS 0
-#endif
-
 // Streaming multiprocessors of the current device (152 on GB300), asked once
 // per device.
 int sm_count()
@@ -791,333 +752,6 @@ int sm_count()
     }
     if (dev >= 0 && dev < 64) cached[dev].store(sms, std::memory_order_relaxed);
     return sms;
-}
-
-// The z run of the streaming convolutions: each CTA walks zrun planes of an
-// 8 x 16 column, xy columns in all, `slots` CTAs resident at once.  A run
-// costs about zrun + 3 planes (the CTA's weights, two halo planes, the
-// pipeline fill), and CTAs beyond the resident ones wait for whole runs, so
-// the run minimises waves x (zrun + 3), longer runs among equals.  At 64^3
-// x 4 samples this takes 512 CTAs of 16 planes in one wave; the earlier rule
-// (about 4 CTAs per SM) gave 640 CTAs of 13 planes, 32 of them in a second
-// wave, and the layer took almost two runs' time.
-int conv_zrun(long long xy, int n, int slots)
-{
-    int best = n, best_cost = 0x7fffffff;
-    for (int zs = 1; zs <= std::max(1, n / 2); ++zs) {
-        const int zrun = (n + zs - 1) / zs;
-        const long long ctas = xy * ((n + zrun - 1) / zrun);
-        const long long waves = (ctas + slots - 1) / slots;
-        const long long cost = waves * (zrun + 3);
-        if (cost < best_cost || (cost == best_cost && zrun > best)) best = zrun, best_cost = static_cast<int>(cost);
-    }
-    return best;
-}
-
-template <int CO, typename TO>
-__global__ void __launch_bounds__(128, 1) conv3d_umma_kernel(const __nv_bfloat16 *__restrict__ x,
-                                                             const __nv_bfloat16 *__restrict__ w,
-                                                             const float *__restrict__ bias,
-                                                             TO *__restrict__ y, int n, int cin, int cout,
-                                                             int act, int *err)
-{
-    extern __shared__ __align__(1024) unsigned char um_smem[];
-    uint64_t *bar = reinterpret_cast<uint64_t *>(um_smem);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(um_smem + 8);
-    unsigned char *halo = um_smem + kUmHaloOff;
-    unsigned char *wsm = halo + kUmHaloBytes;
-    constexpr uint32_t kCols = DMRT_UMMA_TMEM_COLS > (CO < 32 ? 32 : CO) ? DMRT_UMMA_TMEM_COLS : (CO < 32 ? 32 : CO);
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int tx_n = n / kUmX, ty_n = n / kUmY;
-    int r = blockIdx.x;
-    const int x0 = (r % tx_n) * kUmX;
-    r /= tx_n;
-    const int y0 = (r % ty_n) * kUmY;
-    r /= ty_n;
-    const int z = r % n;
-    const int b = r / n;
-    const int co0 = blockIdx.y * CO;
-    const long long sample = static_cast<long long>(b) * n * n * n;
-    if (t == 0) umma::mbar_init(bar, 1);
-    if (warp == 0) umma::tmem_alloc(tslot, kCols);
-    umma::fence_before_sync();
-    __syncthreads();
-    umma::fence_after_sync();
-    const uint32_t tmem = *tslot;
-    constexpr uint32_t idesc = umma::idesc_bf16_f32(128, CO);
-    const uint32_t halo_s = umma::smem_u32(halo), w_s = umma::smem_u32(wsm);
-    const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-    bool ok = true;
-    uint32_t phase = 0;
-    for (int ci0 = 0; ci0 < cin && ok; ci0 += 16) {
-        for (int e = t; e < kUmHalo * 2; e += 128) {
-            const int kg = e / kUmHalo, h = e % kUmHalo;
-            const int hx = h % kUmHX, hy = (h / kUmHX) % kUmHY, hz = h / (kUmHX * kUmHY);
-            const int gx = x0 + hx - 1, gy = y0 + hy - 1, gz = z + hz - 1;
-            const int c = ci0 + 8 * kg;
-            uint4 v = zero4;
-            if (gx >= 0 && gx < n && gy >= 0 && gy < n && gz >= 0 && gz < n && c < cin)
-                v = *reinterpret_cast<const uint4 *>(
-                    x + (sample + (static_cast<long long>(gz) * n + gy) * n + gx) * cin + c);
-            *reinterpret_cast<uint4 *>(halo + (kg * kUmHalo + h) * 16) = v;
-        }
-        for (int e = t; e < 27 * 2 * CO; e += 128) {
-            const int co = e % CO, kg = (e / CO) % 2, tap = e / (2 * CO);
-            const int c = ci0 + 8 * kg;
-            uint4 v = zero4;
-            if (co0 + co < cout && c < cin)
-                v = *reinterpret_cast<const uint4 *>(w + (static_cast<long long>(tap) * cout + co0 + co) * cin + c);
-            *reinterpret_cast<uint4 *>(wsm + ((tap * 2 + kg) * CO + co) * 16) = v;
-        }
-        umma::fence_proxy_async_smem();
-        umma::fence_before_sync();
-        __syncthreads();
-        if (t == 0) {
-            umma::fence_after_sync();
-            for (int tap = 0; tap < 27; ++tap) {
-                const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-                const uint64_t ad = umma::smem_desc(halo_s + ((dz * kUmHY + dy) * kUmHX + dx) * 16,
-                                                    kUmHalo * 16, kUmHX * 16);
-                const uint64_t bd = umma::smem_desc(w_s + tap * 2 * CO * 16, CO * 16, 128);
-                umma::mma_bf16(tmem, ad, bd, idesc, (ci0 > 0 || tap > 0) ? 1u : 0u);
-            }
-            umma::commit(bar);
-        }
-        // the MMAs read the staged tiles: wait for them before restaging
-        if (!umma::mbar_wait(bar, phase, kUmWaitPolls)) ok = false;
-        phase ^= 1u;
-        umma::fence_after_sync();
-        __syncthreads();
-    }
-    if (ok) {
-        const int m = 32 * warp + lane;  // TMEM lane = GEMM row = voxel (x fastest)
-        const long long vox = sample + (static_cast<long long>(z) * n + y0 + m / kUmX) * n + x0 + m % kUmX;
-        TO *yo = y + vox * cout + co0;
-#pragma unroll
-        for (int c16 = 0; c16 < CO; c16 += 16) {
-            float v[16];
-            umma::ld_32x32b_x16(tmem + (static_cast<uint32_t>(32 * warp) << 16) + c16, v);
-#pragma unroll
-            for (int j = 0; j < 16; j += 2) {
-                const int co = co0 + c16 + j;
-                float a = v[j] + (bias ? bias[co] : 0.f), bb = v[j + 1] + (bias ? bias[co + 1] : 0.f);
-                if (act) {
-                    a = a > 0.f ? a : kSlope * a;
-                    bb = bb > 0.f ? bb : kSlope * bb;
-                }
-                st2(yo + c16 + j, a, bb);
-            }
-        }
-    } else if (t == 0) {
-        atomicExch(err, 1);
-    }
-    umma::fence_before_sync();
-    __syncthreads();
-    if (warp == 0) umma::tmem_dealloc(tmem, kCols);
-}
-
-// 3^3 convolution on the tcgen05 tensor cores for few channels (cin <= 32,
-// cout <= 32), streamed along z with its halo planes brought in by TMA and
-// its roles split among warps.  A CTA owns an 8 x 16 tile (M = 128 GEMM
-// rows, one per voxel) over a run of z-planes and keeps the weights of all
-// taps resident in the layout of conv3d_umma_kernel ([tap][kg][co] x 16 B);
-// tap (dz, dy, dx) of plane z is the halo descriptor of plane z - 1 + dz
-// shifted by (dy * 10 + dx) * 16 bytes.
-//  - the halo planes (10 x 18 voxels, 8 channels per k-group) arrive by
-//    tiled TMA copies of the channels-last activations, viewed as the 5-D
-//    tensor (c, x, y, z, sample): one box of 8 x 10 x 18 x 1 x 1 per k-group,
-//    zero-filled outside the grid, into a ring of kUtRing plane slots with
-//    one mbarrier each;
-//  - warp 4 is the producer: one lane issues the copies and the 27 MMAs of a
-//    plane into one of kUtAcc TMEM accumulators, and refills a ring slot as
-//    soon as the MMAs that read it have completed;
-//  - warps 0-3 are the epilogue (TMEM lanes 32 w .. 32 w + 31, one voxel
-//    each): they wait for a plane's MMAs, read its accumulator, hand it back
-//    on an mbarrier and write bias + activation.
-// No thread waits at a block barrier inside the loop: the tensor cores, the
-// copies and the epilogue run concurrently.  What bounds the narrow layers
-// then is the tensor core's operand traffic: each of the 27 MMAs of a plane
-// reads its 128 x 16 A tile (4 KB) from shared memory for only 16 or 32
-// output channels.  Each k-group of a plane starts on a 128-byte boundary
-// (2944 bytes apart), which the MMA descriptors take as the leading byte
-// offset.  Every wait is bounded; one that runs out sets *err and ends its
-// warp's loop, and the CTA waits (bounded) for its copies in flight before it
-// releases its TMEM and exits.
-constexpr int kUtRing = 6;
-constexpr int kUtAcc = 4;  // TMEM accumulators
-constexpr int kUtThreads = 160;
-constexpr unsigned kUtKgBytes = (kUmHX * kUmHY * 16u + 127u) / 128u * 128u;  // 2944
-constexpr unsigned kUtHead = 256;  // mbarriers and the TMEM slot
-template <int KG>
-constexpr unsigned ut_plane_bytes()
-{
-    return static_cast<unsigned>(KG) * kUtKgBytes;
-}
-template <int CO, int KG>
-constexpr unsigned ut_smem_bytes()
-{
-    return 128u + kUtHead + kUtRing * ut_plane_bytes<KG>() + 27u * KG * CO * 16u;  // + alignment slack
-}
-
-template <int CO, int KG, typename TO>
-__global__ void __launch_bounds__(kUtThreads, 4) conv3d_umma_tma_kernel(const __grid_constant__ CUtensorMap xmap,
-                                                                     const __nv_bfloat16 *__restrict__ w,
-                                                                     const float *__restrict__ bias,
-                                                                     TO *__restrict__ y, int n, int cin, int cout,
-                                                                     int act, int zrun, int *err)
-{
-    extern __shared__ __align__(1024) unsigned char ut_smem_raw[];
-    // TMA destinations start on 128-byte boundaries whatever the base alignment
-    unsigned char *ut_smem = ut_smem_raw + ((128u - (umma::smem_u32(ut_smem_raw) & 127u)) & 127u);
-    uint64_t *full = reinterpret_cast<uint64_t *>(ut_smem);  // [kUtRing]: a slot holds its plane
-    uint64_t *acc_full = full + kUtRing;                      // [kUtAcc]: a plane's MMAs are done
-    uint64_t *acc_empty = acc_full + kUtAcc;                  // [kUtAcc]: its accumulator was read
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(acc_empty + kUtAcc);
-    unsigned char *ring = ut_smem + kUtHead;
-    constexpr unsigned kPlane = ut_plane_bytes<KG>();
-    unsigned char *wsm = ring + kUtRing * kPlane;
-    constexpr int kRow = kUmHX * kUmHY;  // 180 voxels of a halo plane
-    constexpr uint32_t kPlaneTx = static_cast<uint32_t>(KG) * kRow * 16u;
-    constexpr uint32_t kCols = kUtAcc * CO < 32 ? 32 : kUtAcc * CO;
-    static_assert(kUtHead >= 8 * (kUtRing + 2 * kUtAcc) + 4, "mbarriers and TMEM slot");
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int tx_n = n / kUmX, ty_n = n / kUmY, zs_n = (n + zrun - 1) / zrun;
-    int r = blockIdx.x;
-    const int x0 = (r % tx_n) * kUmX;
-    r /= tx_n;
-    const int y0 = (r % ty_n) * kUmY;
-    r /= ty_n;
-    const int z_begin = (r % zs_n) * zrun;
-    const int b = r / zs_n;
-    const int z_end = min(z_begin + zrun, n);
-    const long long sample = static_cast<long long>(b) * n * n * n;
-    const int p0 = z_begin - 1;  // the first halo plane; the last one is z_end
-    const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-    if (t == 0) {
-        for (int k = 0; k < kUtRing; ++k) umma::mbar_init(&full[k], 1);
-        for (int k = 0; k < kUtAcc; ++k) {
-            umma::mbar_init(&acc_full[k], 1);
-            umma::mbar_init(&acc_empty[k], 4);  // one arrival per epilogue warp
-        }
-    }
-    if (warp == 0) umma::tmem_alloc(tslot, kCols);
-    // weights of all taps: [tap][kg][co] x 16 B
-    for (int e = t; e < 27 * KG * CO; e += kUtThreads) {
-        const int co = e % CO, kg = (e / CO) % KG, tap = e / (KG * CO);
-        const int c = 8 * kg;
-        uint4 v = zero4;
-        if (co < cout && c < cin)
-            v = *reinterpret_cast<const uint4 *>(w + (static_cast<long long>(tap) * cout + co) * cin + c);
-        *reinterpret_cast<uint4 *>(wsm + ((tap * KG + kg) * CO + co) * 16) = v;
-    }
-    umma::fence_proxy_async_smem();
-    umma::fence_before_sync();
-    __syncthreads();
-    umma::fence_after_sync();
-    const uint32_t tmem = *tslot;
-    bool ok = true;
-    if (warp == 4) {
-        // ---- producer: copies and MMAs (one lane)
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma::idesc_bf16_f32(128, CO);
-            const uint64_t a_base = umma::smem_desc(umma::smem_u32(ring), kUtKgBytes, kUmHX * 16);
-            const uint64_t b_base = umma::smem_desc(umma::smem_u32(wsm), CO * 16, 128);
-            // plane p (p0 <= p <= z_end) is load number (p - p0) / kUtRing of slot (p - p0) % kUtRing
-            auto issue = [&](int p) {
-                const int k = p - p0, slot = k % kUtRing;
-                umma::mbar_arrive_expect_tx(&full[slot], kPlaneTx);
-#pragma unroll
-                for (int kg = 0; kg < KG; ++kg)
-                    umma::tma_load_5d(&xmap, ring + slot * kPlane + kg * kUtKgBytes, &full[slot], 8 * kg, x0 - 1,
-                                      y0 - 1, p, b);
-            };
-            auto wait_plane = [&](int p) {
-                const int k = p - p0;
-                return umma::mbar_wait(&full[k % kUtRing], static_cast<uint32_t>(k / kUtRing) & 1u, kUmWaitPolls);
-            };
-            int issued = p0 - 1;  // the last plane whose copies went out
-            while (issued < z_end && issued + 1 - p0 < kUtRing) issue(++issued);
-            for (int z = z_begin; z < z_end && ok; ++z) {
-                const int j = z - z_begin, buf = j % kUtAcc;
-                // the accumulator's previous plane has been read out
-                if (j >= kUtAcc)
-                    ok = umma::mbar_wait(&acc_empty[buf], static_cast<uint32_t>(j / kUtAcc - 1) & 1u, kUmWaitPolls);
-                ok = ok && wait_plane(z - 1) && wait_plane(z) && wait_plane(z + 1);
-                if (!ok) break;
-                umma::fence_after_sync();
-                // descriptors: the base ones plus each operand's offset / 16 in
-                // the start-address field (shared addresses stay below 2^18)
-                uint64_t a_plane[3];
-#pragma unroll
-                for (int dz = 0; dz < 3; ++dz)
-                    a_plane[dz] = a_base + static_cast<uint64_t>((((z - 1 + dz - p0) % kUtRing) * kPlane) >> 4);
-                const uint32_t dacc = tmem + buf * CO;
-#pragma unroll
-                for (int tap = 0; tap < 27; ++tap) {
-                    const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-#pragma unroll
-                    for (int kc = 0; kc < KG / 2; ++kc) {
-                        const uint64_t ad =
-                            a_plane[dz] + static_cast<uint64_t>(((dy * kUmHX + dx) * 16 + 2 * kc * kUtKgBytes) >> 4);
-                        const uint64_t bd = b_base + static_cast<uint64_t>(((tap * KG + 2 * kc) * CO * 16) >> 4);
-                        umma::mma_bf16(dacc, ad, bd, idesc, (tap > 0 || kc > 0) ? 1u : 0u);
-                    }
-                }
-                umma::commit(&acc_full[buf]);
-                // plane z - 1's MMAs were the last to read the slot of plane z - 2
-                if (j >= 1 && issued < z_end) {
-                    const int jp = j - 1;
-                    ok = umma::mbar_wait(&acc_full[jp % kUtAcc], static_cast<uint32_t>(jp / kUtAcc) & 1u,
-                                         kUmWaitPolls);
-                    if (ok) issue(++issued);
-                }
-            }
-            if (!ok) {
-                atomicExch(err, 1);
-                // copies still in flight land before the CTA's shared memory is released
-                for (int p = max(p0, issued - kUtRing + 1); p <= issued; ++p) (void)wait_plane(p);
-            }
-        }
-    } else {
-        // ---- epilogue: warp w holds TMEM lanes 32 w .. 32 w + 31 (voxel m, x fastest)
-        const int m = 32 * warp + lane;
-        float bv[CO];  // the biases, read once
-#pragma unroll
-        for (int co = 0; co < CO; ++co) bv[co] = bias ? bias[co] : 0.f;
-        for (int z = z_begin; z < z_end && ok; ++z) {
-            const int j = z - z_begin, buf = j % kUtAcc;
-            ok = umma::mbar_wait(&acc_full[buf], static_cast<uint32_t>(j / kUtAcc) & 1u, kUmWaitPolls);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            umma::fence_after_sync();
-            float v[CO];
-#pragma unroll
-            for (int c16 = 0; c16 < CO; c16 += 16) {
-                float part[16];
-                umma::ld_32x32b_x16(tmem + (static_cast<uint32_t>(32 * warp) << 16) + buf * CO + c16, part);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[c16 + i] = part[i];
-            }
-            // the accumulator may take the next plane's MMAs
-            umma::fence_before_sync();
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(umma::smem_u32(&acc_empty[buf]))
-                                        : "memory");
-            const long long vox = sample + (static_cast<long long>(z) * n + y0 + m / kUmX) * n + x0 + m % kUmX;
-            TO *yo = y + vox * cout;
-#pragma unroll
-            for (int co = 0; co < CO; ++co) {
-                const float a = v[co] + bv[co];
-                v[co] = act && a <= 0.f ? kSlope * a : a;
-            }
-#pragma unroll
-            for (int co = 0; co < CO; co += 8) st8(yo + co, v + co);
-        }
-        if (!ok && lane == 0) atomicExch(err, 1);
-    }
-    umma::fence_before_sync();
-    __syncthreads();
-    if (warp == 0) umma::tmem_dealloc(tmem, kCols);
 }
 
 // out = bfloat16(in)
@@ -1699,36 +1333,6 @@ __global__ void target_kernel(const float *__restrict__ u, const float *__restri
     }
 }
 
-// Device word counting tcgen05 waits that ran out (see conv3d_umma_kernel).
-__device__ int g_umma_err;
-
-int *umma_error_word()
-{
-    void *p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_umma_err) != cudaSuccess) return nullptr;
-    return static_cast<int *>(p);
-}
-
-// The tcgen05 convolution is used unless DMRT_NN_NO_TCGEN05 is set in the
-// environment (read once).
-bool umma_enabled()
-{
-    static const bool on = std::getenv("DMRT_NN_NO_TCGEN05") == nullptr;
-    return on;
-}
-
-// Dynamic shared memory of conv3d_umma_kernel<CO>.  DMRT_UMMA_SMEM (bytes)
-// overrides it with a larger allocation.
-#ifndef DMRT_UMMA_SMEM
-#define DMRT_UMMA_SMEM 0
-#endif
-template <int CO>
-unsigned umma_smem()
-{
-    const unsigned need = um_smem_bytes<CO>();
-    return DMRT_UMMA_SMEM > need ? DMRT_UMMA_SMEM : need;
-}
-
 // Elements per block of sum_chunks_kernel and its grid: one thread per
 // element when there are few chunks, else 32 elements (fewer when len is
 // smaller) with the remaining threads as lanes over the chunks.
@@ -1753,45 +1357,9 @@ unsigned flat_blocks(long long len)
     return static_cast<unsigned>(b);
 }
 
-// Tensor map of a channels-last bf16 activation tensor [batch][n][n][n][cin]
-// as the 5-D (c, x, y, z, sample) tensor conv3d_umma_tma_kernel loads its
-// halo planes from: boxes of 8 channels x 10 x 18 x 1 x 1, zeros outside.
-// False if the driver's encoder is missing or rejects the shape.
-bool encode_act_map(const void *x, int batch, int n, int cin, CUtensorMap *map)
-{
-    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    if (!encode) {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess || !fn)
-            return false;
-        encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
-    const cuuint64_t N = static_cast<cuuint64_t>(n), C = static_cast<cuuint64_t>(cin);
-    const cuuint64_t dims[5] = {C, N, N, N, static_cast<cuuint64_t>(batch)};
-    const cuuint64_t strides[4] = {C * 2, N * C * 2, N * N * C * 2, N * N * N * C * 2};
-    const cuuint32_t box[5] = {8, static_cast<cuuint32_t>(kUmHX), static_cast<cuuint32_t>(kUmHY), 1, 1};
-    const cuuint32_t unit[5] = {1, 1, 1, 1, 1};
-    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(x), dims, strides, box, unit,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
-
-int tensor_core_errors(bool reset)
-{
-    int *p = umma_error_word();
-    if (!p) return -1;
-    int v = 0;
-    if (cudaMemcpy(&v, p, sizeof v, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
-    if (reset && cudaMemset(p, 0, sizeof v) != cudaSuccess) return -1;
-    return v;
-}
 
 template <typename TI, typename TW, typename TO>
 cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch, int n, int cin,
@@ -1811,66 +1379,8 @@ cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch
         // channel count and both base pointers must keep 16-byte alignment
         const bool aligned =
             ((reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(w)) & 15ull) == 0;
-        if (k == 3 && aligned && (cin == 8 || cin == 16 || cin == 32) && (cout == 16 || cout == 32) &&
-            n % kUmY == 0 && umma_enabled()) {
-            // stream along z: each CTA walks a run of zrun planes of one 8 x 16
-            // column, the run chosen for the kernel's resident CTAs (conv_zrun)
-            const long long xy = static_cast<long long>(batch) * (n / kUmX) * (n / kUmY);
-            int *err = umma_error_word();
-            if (!err) return cudaErrorInvalidValue;
-            cudaError_t e = cudaSuccess;
-            CUtensorMap xmap;
-            if (encode_act_map(x, batch, n, cin, &xmap)) {
-                // halo planes by TMA
-                auto go_tma = [&](auto kernel, unsigned smem) {
-                    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                    if (e != cudaSuccess) return;
-                    // resident CTAs per SM of this variant: its shared memory
-                    // (plus the 1 KB the runtime reserves per CTA) against the
-                    // SM's 228 KB, at most DMRT_UMMA_CTAS_PER_SM (the launch
-                    // bounds' minimum)
-                    const int per_sm = std::max(
-                        1, std::min(DMRT_UMMA_CTAS_PER_SM, static_cast<int>((228u * 1024u) / (smem + 1024u))));
-                    const int zrun = conv_zrun(xy, n, per_sm * sm_count());
-                    const unsigned grid = static_cast<unsigned>(xy * ((n + zrun - 1) / zrun));
-                    kernel<<<grid, kUtThreads, smem, s>>>(xmap, w, bias, y, n, cin, cout, act, zrun, err);
-                };
-                if (cout == 16 && cin <= 16) go_tma(conv3d_umma_tma_kernel<16, 2, TO>, ut_smem_bytes<16, 2>());
-                else if (cout == 16) go_tma(conv3d_umma_tma_kernel<16, 4, TO>, ut_smem_bytes<16, 4>());
-                else if (cin <= 16) go_tma(conv3d_umma_tma_kernel<32, 2, TO>, ut_smem_bytes<32, 2>());
-                else go_tma(conv3d_umma_tma_kernel<32, 4, TO>, ut_smem_bytes<32, 4>());
-                if (e != cudaSuccess) return e;
-                return cudaGetLastError();
-            }
-            // the driver's encoder rejected the shape: the plane-at-a-time kernel below
-        }
-        if (k == 3 && aligned && (cin == 8 || cin % 16 == 0) && cout % 16 == 0 && n % kUmY == 0 &&
-            umma_enabled()) {
-            const unsigned tiles = static_cast<unsigned>(batch) * (n / kUmX) * (n / kUmY) * n;
-            int *err = umma_error_word();
-            if (!err) return cudaErrorInvalidValue;
-            cudaError_t e;
-            if (cout % 64 == 0) {
-                const unsigned smem = umma_smem<64>();
-                e = cudaFuncSetAttribute(conv3d_umma_kernel<64, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                if (e != cudaSuccess) return e;
-                conv3d_umma_kernel<64, TO><<<dim3(tiles, cout / 64), 128, smem, s>>>(x, w, bias, y, n, cin, cout, act,
-                                                                                   err);
-            } else if (cout % 32 == 0) {
-                const unsigned smem = umma_smem<32>();
-                e = cudaFuncSetAttribute(conv3d_umma_kernel<32, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                if (e != cudaSuccess) return e;
-                conv3d_umma_kernel<32, TO><<<dim3(tiles, cout / 32), 128, smem, s>>>(x, w, bias, y, n, cin, cout, act,
-                                                                                   err);
-            } else {
-                const unsigned smem = umma_smem<16>();
-                e = cudaFuncSetAttribute(conv3d_umma_kernel<16, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                if (e != cudaSuccess) return e;
-                conv3d_umma_kernel<16, TO><<<dim3(tiles, cout / 16), 128, smem, s>>>(x, w, bias, y, n, cin, cout, act,
-                                                                                   err);
-            }
-            return cudaGetLastError();
-        }
+        if (k == 3 && conv3d_umma_takes(x, w, y, batch, n, cin, cout))
+            return conv3d_umma(x, w, bias, y, batch, n, cin, cout, act, s);
         if (k == 3 && aligned && (cin == 8 || cin % 16 == 0) && cout % 16 == 0 && n % kWtX == 0 &&
             n % kWtZ == 0) {
             const unsigned vtiles = static_cast<unsigned>(batch) * (n / kWtX) * (n / kWtY) * (n / kWtZ);

@@ -18,6 +18,14 @@ template <typename TI, typename TW, typename TO>
 cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch, int n, int cin,
                    int cout, int k, int act, cudaStream_t s);
 
+// The 3^3 convolutions of bfloat16 x and w on the tcgen05 tensor cores
+// (conv_umma.cu): taken where the channel counts are multiples of 16 (cin
+// also 8), n a multiple of 8 and the three arrays 16-byte aligned.
+bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout);
+template <typename TO>
+cudaError_t conv3d_umma(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
+                        int cin, int cout, int act, cudaStream_t s);
+
 // dw (FP32, [tap][cout][cin]) of conv3d; scratch holds the per-chunk partials.
 template <typename TI>
 cudaError_t conv3d_wgrad(const TI *x, const float *dy, float *dw, float *scratch,

@@ -139,28 +139,50 @@ __device__ __forceinline__ void fence_proxy_async_smem()
 
 // ---------------------------------------------------------------- MMA
 
-// D[tmem] (+)= A[smem] x B[smem]^T for one K = 16 slice; accumulate = 0
-// overwrites D.  Issued by one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate)
+// True in one lane of the (converged) warp.
+__device__ __forceinline__ uint32_t elect_one()
 {
+    uint32_t e;
     asm volatile(
         "{\n"
         ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(e));
+    return e;
+}
+
+// D[tmem] (+)= A[smem] x B[smem]^T for one K = 16 slice; accumulate = 0
+// overwrites D.  The whole warp executes it and the lane with leader != 0
+// issues it: with every lane on the same path the descriptors stay on the
+// uniform datapath, where the instruction reads them.  Issued from a branch
+// of one lane, each MMA waited for its operands to be moved there.
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                         uint32_t accumulate, uint32_t leader)
+{
+    asm volatile(
+        "{\n"
+        ".reg .pred p, e;\n"
         "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        "setp.ne.b32 e, %5, 0;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
         "}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
         : "memory");
 }
 
-// Arrive on the mbarrier once all previously issued MMAs of this thread
-// have completed.
-__device__ __forceinline__ void commit(uint64_t *bar)
+// Arrive on the mbarrier once all previously issued MMAs of the leader have
+// completed (executed by the whole warp, as the MMAs).
+__device__ __forceinline__ void commit(uint64_t *bar, uint32_t leader)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     smem_u32(bar))
-                 : "memory");
+    asm volatile(
+        "{\n"
+        ".reg .pred e;\n"
+        "setp.ne.b32 e, %1, 0;\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(smem_u32(bar)), "r"(leader)
+        : "memory");
 }
 
 // 16 consecutive FP32 columns of this thread's TMEM lane (warp w reads lanes
