@@ -1042,14 +1042,40 @@ __device__ __forceinline__ void st4<__nv_bfloat16>(__nv_bfloat16 *p, const F4 &f
 
 // Element i of a [batch][n][n][n][c] tensor handled as (voxel, group of 4
 // channels): i = voxel * c4 + q.  Voxel coordinates from the flat index.
+// 32-bit divisions where they suffice: with 64-bit
+// ones the kernels below were bound by them (up2_add at 64^3 x 4, 16
+// channels: UP64 against UP32 us).
 __device__ __forceinline__ void voxel_xyz(long long v, int n, int &x, int &y, int &z, long long &b)
 {
+    if (v < (1LL << 32)) {
+        unsigned u = static_cast<unsigned>(v), d = static_cast<unsigned>(n);
+        x = static_cast<int>(u % d);
+        u /= d;
+        y = static_cast<int>(u % d);
+        u /= d;
+        z = static_cast<int>(u % d);
+        b = u / d;
+        return;
+    }
     x = static_cast<int>(v % n);
     v /= n;
     y = static_cast<int>(v % n);
     v /= n;
     z = static_cast<int>(v % n);
     b = v / n;
+}
+
+// i / d and i % d, in 32 bits where i fits.
+__device__ __forceinline__ long long div_mod(long long i, int d, int &rem)
+{
+    if (i < (1LL << 32)) {
+        const unsigned u = static_cast<unsigned>(i), q = u / static_cast<unsigned>(d);
+        rem = static_cast<int>(u - q * static_cast<unsigned>(d));
+        return q;
+    }
+    const long long q = i / d;
+    rem = static_cast<int>(i - q * d);
+    return q;
 }
 
 // 2 x 2 x 2 average pooling, n -> n / 2 (channels in groups of 4)
@@ -1060,10 +1086,10 @@ __global__ void avgpool2_kernel(const T *__restrict__ x, T *__restrict__ y, int 
     const long long len = static_cast<long long>(batch) * m * m * m * c4;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int q = static_cast<int>(i % c4);
-        int ox, oy, oz;
+        int q, ox, oy, oz;
         long long b;
-        voxel_xyz(i / c4, m, ox, oy, oz, b);
+        const long long vox = div_mod(i, c4, q);
+        voxel_xyz(vox, m, ox, oy, oz, b);
         F4 s{{0.f, 0.f, 0.f, 0.f}};
         for (int k = 0; k < 8; ++k) {
             const int zz = 2 * oz + (k >> 2), yy = 2 * oy + ((k >> 1) & 1), xx = 2 * ox + (k & 1);
@@ -1085,10 +1111,10 @@ __global__ void avgpool2_backward_kernel(const float *__restrict__ dy, float *__
     const long long len = static_cast<long long>(batch) * n * n * n * c4;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int q = static_cast<int>(i % c4);
-        int xx, yy, zz;
+        int q, xx, yy, zz;
         long long b;
-        voxel_xyz(i / c4, n, xx, yy, zz, b);
+        const long long vox = div_mod(i, c4, q);
+        voxel_xyz(vox, n, xx, yy, zz, b);
         F4 a = ld4(dy + (((b * m + zz / 2) * m + yy / 2) * m + xx / 2) * c + 4 * q);
 #pragma unroll
         for (int j = 0; j < 4; ++j) a.v[j] *= 0.125f;
@@ -1105,10 +1131,10 @@ __global__ void up2_add_kernel(const T *__restrict__ x, const T *__restrict__ sk
     const long long len = static_cast<long long>(batch) * m * m * m * c4;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int q = static_cast<int>(i % c4);
-        int xx, yy, zz;
+        int q, xx, yy, zz;
         long long b;
-        voxel_xyz(i / c4, m, xx, yy, zz, b);
+        const long long vox = div_mod(i, c4, q);
+        voxel_xyz(vox, m, xx, yy, zz, b);
         F4 v = ld4(x + (((b * n + zz / 2) * n + yy / 2) * n + xx / 2) * c + 4 * q);
         if (skip) {
             const F4 sk = ld4(skip + 4 * i);
@@ -1127,10 +1153,10 @@ __global__ void up2_backward_kernel(const float *__restrict__ dy, float *__restr
     const long long len = static_cast<long long>(batch) * n * n * n * c4;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int q = static_cast<int>(i % c4);
-        int ox, oy, oz;
+        int q, ox, oy, oz;
         long long b;
-        voxel_xyz(i / c4, n, ox, oy, oz, b);
+        const long long vox = div_mod(i, c4, q);
+        voxel_xyz(vox, n, ox, oy, oz, b);
         F4 s{{0.f, 0.f, 0.f, 0.f}};
         for (int k = 0; k < 8; ++k) {
             const int zz = 2 * oz + (k >> 2), yy = 2 * oy + ((k >> 1) & 1), xx = 2 * ox + (k & 1);
@@ -1239,12 +1265,9 @@ __global__ void features_kernel(const double *__restrict__ ra, const int *__rest
     const float h = 1.0f / n;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int b = static_cast<int>(i / vox);
-        int r = static_cast<int>(i - b * vox);
-        const int xx = r % n;
-        r /= n;
-        const int yy = r % n;
-        const int zz = r / n;
+        int xx, yy, zz;
+        long long b;
+        voxel_xyz(i, n, xx, yy, zz, b);
         const int wl = wall[b];
         const F4 lo{{feat_ra[b], wl == 1 ? 1.f : 0.f, wl == 2 ? 1.f : 0.f, wl == 3 ? 1.f : 0.f}};
         const F4 hi{{2.f * (xx + 0.5f) * h - 1.f, 2.f * (yy + 0.5f) * h - 1.f, 2.f * (zz + 0.5f) * h - 1.f,
@@ -1419,6 +1442,31 @@ cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch
     return cudaGetLastError();
 }
 
+int conv3d_wgrad_chunks(const void *x, const void *dy, int batch, int n, int cin, int cout)
+{
+    const unsigned long long bases = reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(dy);
+    if ((bases & 15ull) != 0 || cout % 16 != 0 || (cin != 8 && cin % 16 != 0) || n % kWtX != 0) return 0;
+    const long long blocks_per_chunk = static_cast<long long>(cout / 16) * (cin > 8 ? cin / 16 : 1);
+    const long long tiles = static_cast<long long>(batch) * (n / kWtX) * (n / kWtY) * (n / kWtZ);
+    // one wave of 3 resident blocks per SM: fewer chunks keep the final sum
+    // over chunks short
+    const long long most = std::min((152 * 3 + blocks_per_chunk - 1) / blocks_per_chunk, tiles);
+    const long long per = (tiles + most - 1) / most;
+    return static_cast<int>((tiles + per - 1) / per);
+}
+
+cudaError_t conv3d_wgrad_partials(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *partials, int chunks, int batch,
+                                  int n, int cin, int cout, cudaStream_t s)
+{
+    const int tiles_per_sample = (n / kWtX) * (n / kWtY) * (n / kWtZ);
+    const long long tiles = static_cast<long long>(batch) * tiles_per_sample;
+    const long long per = (tiles + chunks - 1) / chunks;
+    const dim3 grid(static_cast<unsigned>(cout / 16 * (cin > 8 ? cin / 16 : 1)), static_cast<unsigned>(chunks));
+    wgrad_taps_kernel<<<grid, 256, 0, s>>>(x, dy, partials, n, cin, cout, tiles_per_sample, static_cast<int>(tiles),
+                                           static_cast<int>(per));
+    return cudaGetLastError();
+}
+
 cudaError_t conv3d_wgrad_bf16(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *dw, float *scratch,
                               size_t scratch_floats, int batch, int n, int cin, int cout, int k,
                               cudaStream_t s)
@@ -1426,28 +1474,14 @@ cudaError_t conv3d_wgrad_bf16(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, f
     const bool aligned =
         ((reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(dy)) & 15ull) == 0;
     if (cin % 8 != 0 || cout % 8 != 0 || !aligned || (k != 1 && k != 3)) return cudaErrorInvalidValue;
-    if (k == 3 && cout % 16 == 0 && (cin == 8 || cin % 16 == 0) && n % kWtX == 0 && n % kWtZ == 0) {
-        const int ci_tiles = cin > 8 ? cin / 16 : 1;
-        const long long blocks_per_chunk = static_cast<long long>(cout / 16) * ci_tiles;
-        const long long pairs = static_cast<long long>(cin) * cout;
-        const int tiles_per_sample = (n / kWtX) * (n / kWtY) * (n / kWtZ);
-        const long long total_tiles = static_cast<long long>(batch) * tiles_per_sample;
-        // one wave of 3 resident blocks per SM: fewer chunks keep the final
-        // sum over chunks short
-        long long chunks = (152 * 3 + blocks_per_chunk - 1) / blocks_per_chunk;
-        if (chunks > total_tiles) chunks = total_tiles;
-        while (chunks > 1 && static_cast<size_t>(chunks * 27 * pairs) > scratch_floats) chunks /= 2;
-        if (static_cast<size_t>(chunks * 27 * pairs) > scratch_floats) return cudaErrorInvalidValue;
-        const long long per = (total_tiles + chunks - 1) / chunks;
-        chunks = (total_tiles + per - 1) / per;
-        dim3 grid(static_cast<unsigned>(blocks_per_chunk), static_cast<unsigned>(chunks));
-        wgrad_taps_kernel<<<grid, 256, 0, s>>>(x, dy, scratch, n, cin, cout, tiles_per_sample,
-                                               static_cast<int>(total_tiles), static_cast<int>(per));
-        cudaError_t e = cudaGetLastError();
+    int chunks3 = k == 3 ? conv3d_wgrad_chunks(x, dy, batch, n, cin, cout) : 0;
+    if (chunks3 > 0) {
+        const long long len = 27LL * cin * cout;
+        while (chunks3 > 1 && static_cast<size_t>(chunks3 * len) > scratch_floats) chunks3 /= 2;
+        if (static_cast<size_t>(chunks3 * len) > scratch_floats) return cudaErrorInvalidValue;
+        cudaError_t e = conv3d_wgrad_partials(x, dy, scratch, chunks3, batch, n, cin, cout, s);
         if (e != cudaSuccess) return e;
-        const long long len = 27 * pairs;
-        sum_chunks_kernel<<<sum_blocks(len, static_cast<int>(chunks)), 256, 0, s>>>(
-        scratch, dw, len, static_cast<int>(chunks), sum_width(len, static_cast<int>(chunks)));
+        sum_chunks_kernel<<<sum_blocks(len, chunks3), 256, 0, s>>>(scratch, dw, len, chunks3, sum_width(len, chunks3));
         return cudaGetLastError();
     }
     const long long total = static_cast<long long>(batch) * n * n * n;

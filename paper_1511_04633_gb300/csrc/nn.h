@@ -63,6 +63,64 @@ template <typename T>
 cudaError_t act_backward_narrow_bias(const T *yout, float *dy, __nv_bfloat16 *dyn, long long voxels, int cout,
                                      int act, float *db, float *scratch, size_t scratch_floats, cudaStream_t s);
 
+// ---- the fused backward pass of the bf16 network (nn_backward.cu)
+
+constexpr int kGradBlocks = 152 * 4;  // blocks of grad_narrow: chunks of its bias sums
+constexpr int kHeadBlocks = 152 * 2;  // blocks of head_backward
+constexpr int kMaxSums = 40;
+
+// Arrays whose per-chunk partial sums sum_all adds (and the loss).
+struct SumArray {
+    const float *partials;
+    float *out;
+    size_t stride;
+    int len, chunks, width;
+};
+struct SumList {
+    int count = 0;
+    int first[kMaxSums + 1] = {0};  // first block of each array, then the number of blocks
+    SumArray a[kMaxSums];
+    const double *loss_partials = nullptr;
+    double *loss = nullptr;
+    int loss_parts = 0;
+    double loss_scale = 1.0;
+    void add(const float *partials, size_t stride, float *out, int len, int chunks);
+};
+cudaError_t sum_all(const SumList &list, cudaStream_t s);
+
+// Where grad_narrow's gradient comes from.
+enum class GradSource { kPlain, kUp2, kPool };
+cudaError_t grad_narrow(GradSource src, const float *g, const float *h, const __nv_bfloat16 *yout, __nv_bfloat16 *dyn,
+                        long long voxels, int n, int c, float *partials, cudaStream_t s);
+
+// The 16 -> 5 output head (bf16 h and w; y bf16, or its value widened).
+template <typename TO>
+cudaError_t head_forward(const __nv_bfloat16 *h, const __nv_bfloat16 *w, const float *bias, TO *y, long long voxels,
+                         cudaStream_t s);
+
+// The 16 -> 5 output head's backward with the loss; adds its sums to `sums`.
+size_t head_partial_floats();
+cudaError_t head_backward(const __nv_bfloat16 *out, const float *target, const __nv_bfloat16 *h, const __nv_bfloat16 *w,
+                          __nv_bfloat16 *dyn, long long voxels, float *partials, double *loss_partials, float *dw,
+                          float *db, float *db_before, SumList &sums, cudaStream_t s);
+
+// Layers whose weights flip_all transposes, w and wt at the same offsets.
+constexpr int kMaxFlips = 16;
+struct FlipList {
+    int count = 0;
+    int first[kMaxFlips + 1] = {0};  // first element of each layer, then their number
+    long long offset[kMaxFlips];
+    int cin[kMaxFlips], cout[kMaxFlips];
+};
+cudaError_t flip_all(const __nv_bfloat16 *w, __nv_bfloat16 *wt, const FlipList &list, cudaStream_t s);
+
+// The weight gradient of a 3^3 convolution as `chunks` partial sums of
+// [27][cout][cin], to be added by sum_all: conv3d_wgrad_chunks of them, 0
+// where the shape does not take this path (then use conv3d_wgrad_bf16).
+int conv3d_wgrad_chunks(const void *x, const void *dy, int batch, int n, int cin, int cout);
+cudaError_t conv3d_wgrad_partials(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *partials, int chunks, int batch,
+                                  int n, int cin, int cout, cudaStream_t s);
+
 // weights of the transposed convolution (input gradient = conv3d with them)
 template <typename TW>
 cudaError_t flip_transpose(const TW *w, TW *wt, int k, int cout, int cin, cudaStream_t s);

@@ -47,7 +47,7 @@ struct dmrt_surrogate {
     long long nparams = 0;
     float *master = nullptr, *grad = nullptr, *m1 = nullptr, *m2 = nullptr;
     void *wstore = nullptr;  // weights in the storage type
-    void *wt = nullptr;      // transposed weights scratch (largest layer)
+    void *wt = nullptr;      // transposed weights, each layer's at its offset
     // activations (storage type), per sample batch
     void *x0 = nullptr;
     std::vector<void *> a, s, dd, m, h, pin;  // by level (pin: pooled encoder inputs)
@@ -192,8 +192,10 @@ dmrt_status conv_fwd(dmrt_surrogate_t *s, const Layer &L, const void *in, void *
     return DMRT_OK;
 }
 
+// The network's output into s->out, or (wide not null) as floats into `wide`
+// (device memory).
 template <typename T>
-dmrt_status forward(dmrt_surrogate_t *s, int batch)
+dmrt_status forward(dmrt_surrogate_t *s, int batch, float *wide = nullptr)
 {
     dmrt_status st;
     const int D = s->depth;
@@ -216,7 +218,22 @@ dmrt_status forward(dmrt_surrogate_t *s, int batch)
             "up2_add");
         if ((st = conv_fwd<T>(s, dec_h(s, l), s->m[l], s->h[l], batch))) return st;
     }
-    return conv_fwd<T>(s, head(s), s->h[0], s->out, batch);
+    if constexpr (std::is_same_v<T, __nv_bfloat16>) {
+        if (s->ch[0] == 16) {
+            const auto *h = static_cast<const T *>(s->h[0]);
+            const Layer &L = head(s);
+            const long long vox = batch * voxels(s, 0);
+            SCK(s,
+                wide ? lbm::nn::head_forward<float>(h, W<T>(s, L), B(s, L), wide, vox, s->stream)
+                     : lbm::nn::head_forward<T>(h, W<T>(s, L), B(s, L), static_cast<T *>(s->out), vox, s->stream),
+                "head_forward");
+            return DMRT_OK;
+        }
+    }
+    if ((st = conv_fwd<T>(s, head(s), s->h[0], s->out, batch))) return st;
+    if (wide)
+        SCK(s, lbm::nn::widen<T>(static_cast<const T *>(s->out), wide, batch * voxels(s, 0) * kOut, s->stream), "widen");
+    return DMRT_OK;
 }
 
 // Backward through one convolution whose output gradient is gin (FP32,
@@ -291,6 +308,103 @@ dmrt_status conv_bwd(dmrt_surrogate_t *s, const Layer &L, const void *in, const 
     return DMRT_OK;
 }
 
+// Does the bf16 network take the fused backward pass: a 16-channel finest
+// level (the head kernel), every 3^3 weight gradient by voxel tiles, element
+// counts of 32 bits, room for all partial sums?
+bool fused_backward(const dmrt_surrogate_t *s, int batch)
+{
+    if (s->storage != DMRT_STORE_BF16 || s->ch[0] != 16) return false;
+    size_t floats = lbm::nn::head_partial_floats();
+    for (const Layer &L : s->layers) {
+        if (L.k != 3) continue;
+        const int chunks = lbm::nn::conv3d_wgrad_chunks(nullptr, nullptr, batch, edge(s, L.level), L.cin, L.cout);
+        if (chunks == 0) return false;
+        if (batch * voxels(s, L.level) * std::max(L.cin, L.cout) >= (1LL << 31)) return false;
+        floats += static_cast<size_t>(chunks) * 27 * L.cin * L.cout +
+                  static_cast<size_t>(lbm::nn::kGradBlocks) * L.cout;
+    }
+    return floats <= s->scratch_floats;
+}
+
+// The backward pass of the bf16 network with everything between two
+// convolutions fused (nn_backward.cu); same results as forward_backward, the
+// order of the final sums aside.  The forward pass has run.
+dmrt_status backward_fused(dmrt_surrogate_t *s, int batch)
+{
+    using lbm::nn::GradSource;
+    using B16 = __nv_bfloat16;
+    const int D = s->depth;
+    auto act = [](const void *p) { return static_cast<const B16 *>(p); };
+    lbm::nn::FlipList flips;
+    for (size_t k = 1; k + 1 < s->layers.size(); ++k) {  // the first layer has no input gradient
+        const Layer &L = s->layers[k];
+        const int i = flips.count++;
+        flips.offset[i] = L.w_off;
+        flips.cin[i] = L.cin;
+        flips.cout[i] = L.cout;
+        flips.first[i + 1] = flips.first[i] + 27 * L.cin * L.cout;
+    }
+    SCK(s, lbm::nn::flip_all(W<B16>(s, s->layers[0]) - s->layers[0].w_off, static_cast<B16 *>(s->wt), flips, s->stream),
+        "flip_all");
+    lbm::nn::SumList sums;
+    sums.loss = s->dloss;
+    float *next = s->scratch;  // partial sums, one array after another
+    auto take = [&](size_t floats) {
+        float *p = next;
+        next += (floats + 3) / 4 * 4;  // 16-byte aligned
+        return p;
+    };
+    // the bf16 gradient of L's pre-activation into gnarrow, with L's bias sums
+    auto grad = [&](GradSource src, const Layer &L, const float *g, const float *h, const void *outv) -> dmrt_status {
+        float *p = take(static_cast<size_t>(lbm::nn::kGradBlocks) * L.cout);
+        SCK(s,
+            lbm::nn::grad_narrow(src, g, h, act(outv), s->gnarrow, batch * voxels(s, L.level), edge(s, L.level), L.cout, p,
+                                 s->stream),
+            "grad_narrow");
+        sums.add(p, L.cout, s->grad + L.b_off, L.cout, lbm::nn::kGradBlocks);
+        return DMRT_OK;
+    };
+    // L's weight sums and, if gout, its input gradient, from gnarrow
+    auto conv = [&](const Layer &L, const void *in, float *gout) -> dmrt_status {
+        const int e = edge(s, L.level), len = 27 * L.cin * L.cout;
+        const int chunks = lbm::nn::conv3d_wgrad_chunks(in, s->gnarrow, batch, e, L.cin, L.cout);
+        float *p = take(static_cast<size_t>(chunks) * len);
+        SCK(s, lbm::nn::conv3d_wgrad_partials(act(in), s->gnarrow, p, chunks, batch, e, L.cin, L.cout, s->stream),
+            "conv3d_wgrad");
+        sums.add(p, len, s->grad + L.w_off, len, chunks);
+        if (gout)
+            SCK(s,
+                (lbm::nn::conv3d<B16, B16, float>(s->gnarrow, static_cast<const B16 *>(s->wt) + L.w_off, nullptr, gout,
+                                                  batch, e, L.cout, L.cin, 3, 0, s->stream)),
+                "conv3d (input gradient)");
+        return DMRT_OK;
+    };
+    dmrt_status st;
+    const Layer &H = head(s);
+    SCK(s,
+        lbm::nn::head_backward(act(s->out), s->target, act(s->h[0]), W<B16>(s, H), s->gnarrow, batch * voxels(s, 0),
+                               take(lbm::nn::head_partial_floats()), s->dpart, s->grad + H.w_off, s->grad + H.b_off,
+                               s->grad + dec_h(s, 0).b_off, sums, s->stream),
+        "head_backward");
+    for (int l = 0; l < D; ++l) {
+        if (l > 0 && (st = grad(GradSource::kPlain, dec_h(s, l), s->g0, nullptr, s->h[l]))) return st;
+        // h_l = act(conv3(m_l)), m_l = up2(d_l) + s_l: gs[l] is the gradient of both
+        if ((st = conv(dec_h(s, l), s->m[l], s->gs[l]))) return st;
+        if ((st = grad(GradSource::kUp2, dec_d(s, l), s->gs[l], nullptr, s->dd[l]))) return st;
+        if ((st = conv(dec_d(s, l), l + 1 == D ? s->s[D] : s->h[l + 1], s->g0))) return st;
+    }
+    for (int l = D; l >= 0; --l) {
+        st = l == D ? grad(GradSource::kPlain, enc_s(s, l), s->g0, nullptr, s->s[l])
+                    : grad(GradSource::kPool, enc_s(s, l), s->gs[l], s->g0, s->s[l]);
+        if (st) return st;
+        if ((st = conv(enc_s(s, l), s->a[l], s->g1))) return st;
+        if ((st = grad(GradSource::kPlain, enc_a(s, l), s->g1, nullptr, s->a[l]))) return st;
+        if ((st = conv(enc_a(s, l), l == 0 ? s->x0 : s->pin[l], l == 0 ? nullptr : s->g0))) return st;
+    }
+    SCK(s, lbm::nn::sum_all(sums, s->stream), "sum_all");
+    return DMRT_OK;
+}
+
 // Loss and gradients for a batch whose features are in x0 and targets in
 // s->target; leaves d loss / d params in s->grad and the loss in s->dloss.
 template <typename T>
@@ -298,6 +412,8 @@ dmrt_status forward_backward(dmrt_surrogate_t *s, int batch)
 {
     dmrt_status st;
     if ((st = forward<T>(s, batch))) return st;
+    if constexpr (std::is_same_v<T, __nv_bfloat16>)
+        if (fused_backward(s, batch)) return backward_fused(s, batch);
     const int D = s->depth;
     const long long fine = static_cast<long long>(batch) * voxels(s, 0);
     // dout in g0
@@ -410,10 +526,7 @@ dmrt_status dmrt_surrogate_create(dmrt_surrogate_t **out, const dmrt_surrogate_c
               dalloc(reinterpret_cast<void **>(&s->grad), P * 4) &&
               dalloc(reinterpret_cast<void **>(&s->m1), P * 4) && dalloc(reinterpret_cast<void **>(&s->m2), P * 4) &&
               dalloc(&s->wstore, P * es);
-    long long wt_max = 0;
-    for (const Layer &L : s->layers)
-        wt_max = std::max(wt_max, static_cast<long long>(L.k) * L.k * L.k * L.cin * L.cout);
-    ok = ok && dalloc(&s->wt, static_cast<size_t>(wt_max) * es);
+    ok = ok && dalloc(&s->wt, P * es);
     ok = ok && dalloc(&s->x0, static_cast<size_t>(Bm) * voxels(s, 0) * lbm::nn::kFeatures * es);
     s->a.assign(s->depth + 1, nullptr);
     s->s.assign(s->depth + 1, nullptr);
@@ -441,7 +554,18 @@ dmrt_status dmrt_surrogate_create(dmrt_surrogate_t **out, const dmrt_surrogate_c
          dalloc(reinterpret_cast<void **>(&s->g2), gmax * 4) &&
          dalloc(reinterpret_cast<void **>(&s->gnarrow), gmax * 2) &&
          dalloc(reinterpret_cast<void **>(&s->target), static_cast<size_t>(Bm) * voxels(s, 0) * kOut * 4);
+    // partial sums: of one layer, or of all of them (backward_fused)
     s->scratch_floats = std::max<size_t>(static_cast<size_t>(27) * 128 * 128 * 64, 4u << 20);
+    {
+        size_t all = lbm::nn::head_partial_floats() + 64;
+        for (const Layer &L : s->layers)
+            if (L.k == 3)
+                // (the most chunks, which a large batch takes)
+                all += static_cast<size_t>(lbm::nn::conv3d_wgrad_chunks(nullptr, nullptr, 4096, edge(s, L.level), L.cin, L.cout)) *
+                           27 * L.cin * L.cout +
+                       static_cast<size_t>(lbm::nn::kGradBlocks) * L.cout;
+        s->scratch_floats = std::max(s->scratch_floats, all);
+    }
     s->bscratch_floats = static_cast<size_t>(152) * 4 * 128;
     ok = ok && dalloc(reinterpret_cast<void **>(&s->scratch), s->scratch_floats * 4) &&
          dalloc(reinterpret_cast<void **>(&s->bscratch), s->bscratch_floats * 4) &&
@@ -530,15 +654,11 @@ dmrt_status dmrt_surrogate_predict(dmrt_surrogate_t *s, int batch, const double 
         using T = std::remove_pointer_t<decltype(tp)>;
         dmrt_status r = make_features<T>(s, batch, ra, wall);
         if (r != DMRT_OK) return r;
-        r = forward<T>(s, batch);
-        if (r != DMRT_OK) return r;
-        SCK(s, lbm::nn::widen<T>(static_cast<const T *>(s->out), s->g0, len, s->stream), "widen");
-        return DMRT_OK;
+        return forward<T>(s, batch, on_device ? out : s->g0);
     });
     if (st != DMRT_OK) return st;
-    SCK(s, cudaMemcpyAsync(out, s->g0, len * 4, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                           s->stream),
-        "copy prediction");
+    if (!on_device)
+        SCK(s, cudaMemcpyAsync(out, s->g0, len * 4, cudaMemcpyDeviceToHost, s->stream), "copy prediction");
     SCK(s, cudaStreamSynchronize(s->stream), "cudaStreamSynchronize");
     return DMRT_OK;
 }
@@ -638,17 +758,13 @@ dmrt_status dmrt_warm_start(dmrt_t *h, dmrt_surrogate_t *s, double Ra, int wall)
         return sfail(s, DMRT_ERR_ARG, "warm start needs a cubic cavity (got %dx%dx%d)", p.nx, p.ny, p.nz);
     SGuard g(s->device);
     // the prediction at the network grid, FP32 channels-last, in g1
-    const long long len = voxels(s, 0) * kOut;
     st = by_storage(s, [&](auto *tp) -> dmrt_status {
         using T = std::remove_pointer_t<decltype(tp)>;
         dmrt_status r = make_features<T>(s, 1, &Ra, &wall);
         if (r != DMRT_OK) return r;
         r = check_batch(s, 1, &Ra, &wall);
         if (r != DMRT_OK) return r;
-        r = forward<T>(s, 1);
-        if (r != DMRT_OK) return r;
-        SCK(s, lbm::nn::widen<T>(static_cast<const T *>(s->out), s->g1, len, s->stream), "widen");
-        return DMRT_OK;
+        return forward<T>(s, 1, s->g1);
     });
     if (st != DMRT_OK) return st;
     // trilinear resampling to the cavity grid; u scaled back by u_c
