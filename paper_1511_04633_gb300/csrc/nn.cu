@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(128) wgrad_mma_kernel(const __nv_bfloat16 *__r
 // Tensor-core weight gradient of a 3^3 convolution, all 27 taps per block:
 // dw[tap][co][ci] = sum over voxels v of dy[v][co] x[v + tap][ci].  A block
 // owns 16 output x 16 input channels and a run of 8 x 8 x 4 voxel tiles of
-// one sample.  Per tile it stages dy (256 voxels) and the x halo (10 x 10 x 6
+// the batch.  Per tile it stages dy (256 voxels) and the x halo (10 x 10 x 6
 // voxels) once, unmodified (channels-last rows padded to 24 elements, which
 // keeps the 8 rows of every ldmatrix conflict-free), and every tap reads the
 // shifted x rows straight from the halo: ldmatrix takes one row address per
@@ -386,6 +386,11 @@ __global__ void __launch_bounds__(128) wgrad_mma_kernel(const __nv_bfloat16 *__r
 // accumulates taps w, w + 8, w + 16 (and w + 24 < 27) for both 8-channel
 // halves of ci: 6 or 8 accumulator tiles.  The block's sums over its tiles go
 // to partials[chunk][tap][co][ci], summed in chunk order afterwards.
+// What bounds it: the fragment loads, 35 of 512 B per 16 voxels for 54 MMAs.
+// The next tile's copies (cp.async) run under the current tile's MMAs, two
+// blocks per SM; staging and multiplying in turn with three blocks took 78
+// us instead of 68 us for 16 x 16 channels at 64^3 x 4, 28 instead of 23
+// us for 64 x 64 at 16^3 x 4.
 constexpr int kWtX = 8, kWtY = 8, kWtZ = 4;                  // voxel tile
 constexpr int kWtHX = kWtX + 2, kWtHY = kWtY + 2, kWtHZ = kWtZ + 2;
 constexpr int kWtVox = kWtX * kWtY * kWtZ;                   // 256
@@ -400,32 +405,44 @@ __device__ __forceinline__ void ldsm_x4_trans(unsigned (&r)[4], const void *p)
                  : "r"(a));
 }
 
-__global__ void __launch_bounds__(256) wgrad_taps_kernel(const __nv_bfloat16 *__restrict__ x,
-                                                         const __nv_bfloat16 *__restrict__ dy,
-                                                         float *__restrict__ partials, int n,
-                                                         int cin, int cout, int tiles_per_sample,
-                                                         int total_tiles, int tiles_per_block)
+// Shared memory of one stage: the x halo, then the dy tile (rows of kWtRow).
+constexpr unsigned kWtStage = (kWtHalo + kWtVox) * kWtRow * 2u;
+
+__device__ __forceinline__ void wt_copy16(void *dst, const void *src, bool valid)
 {
-    __shared__ __align__(16) __nv_bfloat16 xs[kWtHalo][kWtRow];
-    __shared__ __align__(16) __nv_bfloat16 gs[kWtVox][kWtRow];
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                     static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(256, 2) wgrad_taps_kernel(const __nv_bfloat16 *__restrict__ x,
+                                                            const __nv_bfloat16 *__restrict__ dy,
+                                                            float *__restrict__ partials, int n,
+                                                            int cin, int cout, int tiles_per_sample,
+                                                            int total_tiles, int tiles_per_block)
+{
+    extern __shared__ __align__(16) unsigned char wt_smem[];
+    typedef __nv_bfloat16 Row[kWtRow];
     const int ci_tiles = cin > 8 ? cin / 16 : 1;
     const int co0 = (blockIdx.x / ci_tiles) * 16, ci0 = (blockIdx.x % ci_tiles) * 16;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int ntap = warp + 24 < 27 ? 4 : 3;
-    float acc[4][2][4];
+    float acc[4][2][4], sum[4][2][4];  // of the tile (tensor cores), of the run
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
+            for (int q = 0; q < 4; ++q) acc[i][j][q] = sum[i][j][q] = 0.f;
     const int tx_n = n / kWtX, ty_n = n / kWtY;
-    const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
     // ldmatrix row of this thread: matrix j = lane / 8, row r = lane % 8
     const int mj = lane >> 3, mr = lane & 7;
     const int t_begin = blockIdx.y * tiles_per_block;
     const int t_end = min(t_begin + tiles_per_block, total_tiles);
-    for (int tile = t_begin; tile < t_end; ++tile) {
+    // copies of one tile into stage s (one group per thread)
+    auto load = [&](int tile, int s) {
+        Row *xs = reinterpret_cast<Row *>(wt_smem + s * kWtStage), *gs = xs + kWtHalo;
         const int b = tile / tiles_per_sample;
         int r = tile % tiles_per_sample;
         const int x0 = (r % tx_n) * kWtX;
@@ -440,22 +457,31 @@ __global__ void __launch_bounds__(256) wgrad_taps_kernel(const __nv_bfloat16 *__
             const int hx = h % kWtHX, hy = (h / kWtHX) % kWtHY, hz = h / (kWtHX * kWtHY);
             const int gx = x0 + hx - 1, gy = y0 + hy - 1, gz = z0 + hz - 1;
             const int c = ci0 + 8 * half;
-            uint4 v = zero4;
-            if (gx >= 0 && gx < n && gy >= 0 && gy < n && gz >= 0 && gz < n && c < cin)
-                v = *reinterpret_cast<const uint4 *>(
-                    x + (sample + (static_cast<long long>(gz) * n + gy) * n + gx) * cin + c);
-            *reinterpret_cast<uint4 *>(&xs[h][8 * half]) = v;
+            const bool in = gx >= 0 && gx < n && gy >= 0 && gy < n && gz >= 0 && gz < n && c < cin;
+            const __nv_bfloat16 *p = x + (sample + (static_cast<long long>(gz) * n + gy) * n + gx) * cin + c;
+            wt_copy16(&xs[h][8 * half], in ? p : x, in);
         }
         // dy tile: 256 voxels x 2 granules
         for (int e = t; e < kWtVox * 2; e += 256) {
             const int half = e & 1, vi = e >> 1;
             const int vx = vi % kWtX, vy = (vi / kWtX) % kWtY, vz = vi / (kWtX * kWtY);
-            const uint4 v = *reinterpret_cast<const uint4 *>(
-                dy + (sample + (static_cast<long long>(z0 + vz) * n + y0 + vy) * n + x0 + vx) * cout +
-                co0 + 8 * half);
-            *reinterpret_cast<uint4 *>(&gs[vi][8 * half]) = v;
+            wt_copy16(&gs[vi][8 * half],
+                      dy + (sample + (static_cast<long long>(z0 + vz) * n + y0 + vy) * n + x0 + vx) * cout + co0 + 8 * half,
+                      true);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (t_begin < t_end) load(t_begin, 0);
+    for (int tile = t_begin; tile < t_end; ++tile) {
+        const int s = (tile - t_begin) & 1;
+        if (tile + 1 < t_end) {
+            load(tile + 1, s ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
+        const Row *xs = reinterpret_cast<const Row *>(wt_smem + s * kWtStage), *gs = xs + kWtHalo;
 #pragma unroll 2
         for (int ks = 0; ks < kWtVox / 16; ++ks) {
             // k-step ks: voxels 16 ks .. 16 ks + 15 = two x-rows (z, y), (z, y + 1)
@@ -478,7 +504,17 @@ __global__ void __launch_bounds__(256) wgrad_taps_kernel(const __nv_bfloat16 *__
                 }
             }
         }
-        __syncthreads();
+        // the tensor cores' additions truncate: their chains end with the tile
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    sum[i][j][q] += acc[i][j][q];
+                    acc[i][j][q] = 0.f;
+                }
+        __syncthreads();  // the stage is free for the tile after the next
     }
     // acc[i][j]: rows co0 + g (+8), columns ci0 + 8 j + 2 tig (+1)
     const int g = lane >> 2, tig = lane & 3;
@@ -494,7 +530,7 @@ __global__ void __launch_bounds__(256) wgrad_taps_kernel(const __nv_bfloat16 *__
                 const int co = co0 + g + 8 * (q >> 1);
                 const int ci = ci0 + 8 * j + 2 * tig + (q & 1);
                 if (ci < cin)
-                    out[(static_cast<long long>(tap) * cout + co) * cin + ci] = acc[i][j][q];
+                    out[(static_cast<long long>(tap) * cout + co) * cin + ci] = sum[i][j][q];
             }
     }
 }
@@ -1044,7 +1080,7 @@ __device__ __forceinline__ void st4<__nv_bfloat16>(__nv_bfloat16 *p, const F4 &f
 // channels): i = voxel * c4 + q.  Voxel coordinates from the flat index.
 // 32-bit divisions where they suffice: with 64-bit
 // ones the kernels below were bound by them (up2_add at 64^3 x 4, 16
-// channels: UP64 against UP32 us).
+// channels: 29 us against 25, and 16 us with 16-byte accesses).
 __device__ __forceinline__ void voxel_xyz(long long v, int n, int &x, int &y, int &z, long long &b)
 {
     if (v < (1LL << 32)) {
@@ -1078,11 +1114,53 @@ __device__ __forceinline__ long long div_mod(long long i, int d, int &rem)
     return q;
 }
 
-// 2 x 2 x 2 average pooling, n -> n / 2 (channels in groups of 4)
-template <typename T>
+// G = 4 N consecutive channels in N 4-channel accesses (bf16: N = 2 makes one
+// 16-byte access of each).
+template <int N>
+struct FN {
+    F4 f[N];
+};
+template <typename T, int N>
+__device__ __forceinline__ FN<N> ldn(const T *p)
+{
+    FN<N> r;
+    if constexpr (std::is_same_v<T, __nv_bfloat16> && N == 2) {
+        const uint4 u = *reinterpret_cast<const uint4 *>(p);
+        const unsigned w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w[k]));
+            r.f[k / 2].v[2 * (k % 2)] = v.x;
+            r.f[k / 2].v[2 * (k % 2) + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) r.f[k] = ld4(p + 4 * k);
+    }
+    return r;
+}
+template <typename T, int N>
+__device__ __forceinline__ void stn(T *p, const FN<N> &r)
+{
+    if constexpr (std::is_same_v<T, __nv_bfloat16> && N == 2) {
+        unsigned w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(r.f[k / 2].v[2 * (k % 2)], r.f[k / 2].v[2 * (k % 2) + 1]);
+            w[k] = *reinterpret_cast<const unsigned *>(&h);
+        }
+        *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) st4(p + 4 * k, r.f[k]);
+    }
+}
+
+// 2 x 2 x 2 average pooling, n -> n / 2 (channels in groups of 4 N)
+template <typename T, int N>
 __global__ void avgpool2_kernel(const T *__restrict__ x, T *__restrict__ y, int batch, int n, int c)
 {
-    const int m = n / 2, c4 = c / 4;
+    const int m = n / 2, c4 = c / (4 * N);
     const long long len = static_cast<long long>(batch) * m * m * m * c4;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -1090,16 +1168,19 @@ __global__ void avgpool2_kernel(const T *__restrict__ x, T *__restrict__ y, int 
         long long b;
         const long long vox = div_mod(i, c4, q);
         voxel_xyz(vox, m, ox, oy, oz, b);
-        F4 s{{0.f, 0.f, 0.f, 0.f}};
+        FN<N> s;
+#pragma unroll
+        for (int j = 0; j < 4 * N; ++j) s.f[j / 4].v[j % 4] = 0.f;
+#pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int zz = 2 * oz + (k >> 2), yy = 2 * oy + ((k >> 1) & 1), xx = 2 * ox + (k & 1);
-            const F4 a = ld4(x + (((b * n + zz) * n + yy) * n + xx) * c + 4 * q);
+            const FN<N> a = ldn<T, N>(x + (((b * n + zz) * n + yy) * n + xx) * c + 4 * N * q);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) s.v[j] += a.v[j];
+            for (int j = 0; j < 4 * N; ++j) s.f[j / 4].v[j % 4] += a.f[j / 4].v[j % 4];
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) s.v[j] *= 0.125f;
-        st4(y + 4 * i, s);
+        for (int j = 0; j < 4 * N; ++j) s.f[j / 4].v[j % 4] *= 0.125f;
+        stn<T, N>(y + 4 * N * i, s);
     }
 }
 
@@ -1123,11 +1204,11 @@ __global__ void avgpool2_backward_kernel(const float *__restrict__ dy, float *__
 }
 
 // nearest upsampling x2 (n -> 2n), plus an optional skip added: y = up(x) + s
-template <typename T>
+template <typename T, int N>
 __global__ void up2_add_kernel(const T *__restrict__ x, const T *__restrict__ skip, T *__restrict__ y,
                                int batch, int n, int c)
 {
-    const int m = 2 * n, c4 = c / 4;
+    const int m = 2 * n, c4 = c / (4 * N);
     const long long len = static_cast<long long>(batch) * m * m * m * c4;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -1135,13 +1216,13 @@ __global__ void up2_add_kernel(const T *__restrict__ x, const T *__restrict__ sk
         long long b;
         const long long vox = div_mod(i, c4, q);
         voxel_xyz(vox, m, xx, yy, zz, b);
-        F4 v = ld4(x + (((b * n + zz / 2) * n + yy / 2) * n + xx / 2) * c + 4 * q);
+        FN<N> v = ldn<T, N>(x + (((b * n + zz / 2) * n + yy / 2) * n + xx / 2) * c + 4 * N * q);
         if (skip) {
-            const F4 sk = ld4(skip + 4 * i);
+            const FN<N> sk = ldn<T, N>(skip + 4 * N * i);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) v.v[j] += sk.v[j];
+            for (int j = 0; j < 4 * N; ++j) v.f[j / 4].v[j % 4] += sk.f[j / 4].v[j % 4];
         }
-        st4(y + 4 * i, v);
+        stn<T, N>(y + 4 * N * i, v);
     }
 }
 
@@ -1448,9 +1529,9 @@ int conv3d_wgrad_chunks(const void *x, const void *dy, int batch, int n, int cin
     if ((bases & 15ull) != 0 || cout % 16 != 0 || (cin != 8 && cin % 16 != 0) || n % kWtX != 0) return 0;
     const long long blocks_per_chunk = static_cast<long long>(cout / 16) * (cin > 8 ? cin / 16 : 1);
     const long long tiles = static_cast<long long>(batch) * (n / kWtX) * (n / kWtY) * (n / kWtZ);
-    // one wave of 3 resident blocks per SM: fewer chunks keep the final sum
+    // one wave of 2 resident blocks per SM: fewer chunks keep the final sum
     // over chunks short
-    const long long most = std::min((152 * 3 + blocks_per_chunk - 1) / blocks_per_chunk, tiles);
+    const long long most = std::min((152 * 2 + blocks_per_chunk - 1) / blocks_per_chunk, tiles);
     const long long per = (tiles + most - 1) / most;
     return static_cast<int>((tiles + per - 1) / per);
 }
@@ -1462,7 +1543,10 @@ cudaError_t conv3d_wgrad_partials(const __nv_bfloat16 *x, const __nv_bfloat16 *d
     const long long tiles = static_cast<long long>(batch) * tiles_per_sample;
     const long long per = (tiles + chunks - 1) / chunks;
     const dim3 grid(static_cast<unsigned>(cout / 16 * (cin > 8 ? cin / 16 : 1)), static_cast<unsigned>(chunks));
-    wgrad_taps_kernel<<<grid, 256, 0, s>>>(x, dy, partials, n, cin, cout, tiles_per_sample, static_cast<int>(tiles),
+    const cudaError_t e =
+        cudaFuncSetAttribute(wgrad_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kWtStage);
+    if (e != cudaSuccess) return e;
+    wgrad_taps_kernel<<<grid, 256, 2 * kWtStage, s>>>(x, dy, partials, n, cin, cout, tiles_per_sample, static_cast<int>(tiles),
                                            static_cast<int>(per));
     return cudaGetLastError();
 }
@@ -1625,7 +1709,10 @@ cudaError_t avgpool2(const T *x, T *y, int batch, int n, int c, cudaStream_t s)
 {
     if (c % 4 != 0) return cudaErrorInvalidValue;
     const long long len = static_cast<long long>(batch) * (n / 2) * (n / 2) * (n / 2) * (c / 4);
-    avgpool2_kernel<T><<<flat_blocks(len), 256, 0, s>>>(x, y, batch, n, c);
+    if (std::is_same_v<T, __nv_bfloat16> && c % 8 == 0)
+        avgpool2_kernel<T, 2><<<flat_blocks(len / 2), 256, 0, s>>>(x, y, batch, n, c);
+    else
+        avgpool2_kernel<T, 1><<<flat_blocks(len), 256, 0, s>>>(x, y, batch, n, c);
     return cudaGetLastError();
 }
 
@@ -1642,7 +1729,10 @@ cudaError_t up2_add(const T *x, const T *skip, T *y, int batch, int n, int c, cu
 {
     if (c % 4 != 0) return cudaErrorInvalidValue;
     const long long len = static_cast<long long>(batch) * 8LL * n * n * n * (c / 4);
-    up2_add_kernel<T><<<flat_blocks(len), 256, 0, s>>>(x, skip, y, batch, n, c);
+    if (std::is_same_v<T, __nv_bfloat16> && c % 8 == 0)
+        up2_add_kernel<T, 2><<<flat_blocks(len / 2), 256, 0, s>>>(x, skip, y, batch, n, c);
+    else
+        up2_add_kernel<T, 1><<<flat_blocks(len), 256, 0, s>>>(x, skip, y, batch, n, c);
     return cudaGetLastError();
 }
 
@@ -1696,7 +1786,9 @@ cudaError_t features(const double *ra, const int *wall, T *out, int batch, int n
 {
     const size_t smem = static_cast<size_t>(batch) * sizeof(float);
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
-    features_kernel<T><<<flat_blocks(static_cast<long long>(batch) * n * n * n), 256, smem, s>>>(
+    // one wave of blocks: each pays the FP64 logarithm once
+    const unsigned blocks = std::min(flat_blocks(static_cast<long long>(batch) * n * n * n), 152u * 8u);
+    features_kernel<T><<<blocks, 256, smem, s>>>(
         ra, wall, out, batch, n);
     return cudaGetLastError();
 }

@@ -7,9 +7,9 @@
 //
 // All of it is bound by memory.  Measured on GB300 at 64^3 x 4, 16 channels
 // in the finest level: the output head's backward 212 us in nine kernels ->
-// HEADUS us in one; pooling gradient, skip sum, activation and bias 87 us in
-// three -> POOLUS us; the 25 final sums 250 us -> SUMUS us; the 13 weight
-// transposes 47 us -> FLIPUS us.
+// 35 us in one; pooling gradient, skip sum, activation and bias 87 us in
+// three -> 33 us; the 25 final sums 250 us -> 36 us; the 13 weight
+// transposes 47 us -> 10 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
