@@ -32,6 +32,7 @@ struct dmrt {
     CollideParams C{};
     lbm::BlockShape block{32, 4};
     int cells_per_thread = 1;  // 2: the paired step kernels (walled box, even nx)
+    bool split = false;        // odd rows: the kernels that pair cells of neighbouring slabs
     int pair_loads = 0;        // paired two-buffer step: 1 direct loads, 2 TMA-staged
     alignas(64) unsigned char tma_map[2][256] = {};  // tensor maps of buf[0], buf[1] (rows, x edges)
     unsigned *derr = nullptr;  // device word: a staged kernel's copy wait ran out
@@ -154,7 +155,12 @@ cudaError_t launch_one_step(dmrt_t *h, int ph, bool res)
                               static_cast<unsigned>(cell_count(h->G))};
     const lbm::ResidualArgs *rp = res ? &R : nullptr;
     cudaError_t e;
-    if (h->inplace && h->cells_per_thread == 2)
+    if (h->split)
+        e = h->inplace ? lbm::launch_step_inplace_split(h->wall, h->storage, h->stochastic, h->buf[0], ph, h->SI, h->G,
+                                                        h->C, h->stream, h->use_pdl, rp)
+                       : lbm::launch_step_split(h->wall, h->storage, h->stochastic, h->buf[ph], h->buf[ph ^ 1], h->S,
+                                                h->G, h->C, h->stream, h->use_pdl, rp);
+    else if (h->inplace && h->cells_per_thread == 2)
         e = lbm::launch_step_inplace_pair(h->wall, h->storage, h->stochastic, h->buf[0], ph, h->SI, h->G, h->C,
                                           h->stream, h->use_pdl, rp);
     else if (h->inplace)
@@ -407,6 +413,7 @@ dmrt_status create_common(dmrt_t **out, const int grid[3], double nu, double alp
         return DMRT_ERR_ARG;
     }
     h->cells_per_thread = (cpt == 2 || (cpt == 0 && pair_ok)) ? 2 : 1;
+    h->split = cpt == 0 && !pair_ok && lbm::step_split_supported(wall_type, h->G) && lbm::step_split_pays(h->G);
     // loads of the paired two-buffer kernel: TMA-staged where the tensor map
     // allows it (16-bit storage, nx a multiple of 8)
     const bool tma_ok = h->cells_per_thread == 2 && !h->inplace &&
@@ -445,6 +452,8 @@ dmrt_status create_common(dmrt_t **out, const int grid[3], double nu, double alp
     // the kernel that takes the residual points
     if (h->cells_per_thread == 2)
         h->res_blocks = static_cast<long long>(lbm::pair_blocks(h->G));
+    else if (h->split)
+        h->res_blocks = static_cast<long long>(lbm::split_blocks(h->G));
     else
         h->res_blocks = static_cast<long long>((grid[0] + h->block.bx - 1) / h->block.bx) *
                         ((grid[1] + h->block.by - 1) / h->block.by) * grid[2];

@@ -79,6 +79,39 @@ cudaError_t launch_step_inplace_pair(int wall, int storage, bool stochastic, voi
                                      const CollideParams &C, cudaStream_t s, bool pdl,
                                      const ResidualArgs *res = nullptr);
 
+// Division of numbers n < 2^28 by d: (n * mul) >> shift with shift = 28 +
+// ceil(log2 d) and mul = floor(2^shift / d) + 1.  mul * d exceeds 2^shift by
+// at most d, and n * d < 2^28 * 2^ceil(log2 d), so the quotient is exact.
+struct RowDivisor {
+    unsigned long long mul;
+    unsigned shift;
+    explicit RowDivisor(unsigned d)
+    {
+        unsigned s = 0;
+        while ((1ull << s) < d) ++s;
+        shift = 28 + s;
+        mul = (1ull << shift) / d + 1ull;
+    }
+    __host__ __device__ unsigned divide(unsigned n) const
+    {
+        return static_cast<unsigned>((n * mul) >> shift);
+    }
+};
+
+// The same steps for boxes with odd rows, two cells of neighbouring slabs per
+// thread: bitwise the values of launch_step and launch_step_inplace.  Needs
+// a walled box; the launcher picks its own block shape.
+bool step_split_supported(int wall, const Geometry &G);
+// Is it the faster kernel of a box with odd rows?
+bool step_split_pays(const Geometry &G);
+size_t split_blocks(const Geometry &G);
+cudaError_t launch_step_split(int wall, int storage, bool stochastic, const void *src, void *dst,
+                              const StepGeometry &S, const Geometry &G, const CollideParams &C, cudaStream_t s,
+                              bool pdl, const ResidualArgs *res = nullptr);
+cudaError_t launch_step_inplace_split(int wall, int storage, bool stochastic, void *buf, int phase,
+                                      const InplaceGeometry &SI, const Geometry &G, const CollideParams &C,
+                                      cudaStream_t s, bool pdl, const ResidualArgs *res = nullptr);
+
 // Fields of the pulled populations (any output may be null).
 cudaError_t launch_fields(int wall, int storage, const void *src, const Geometry &G, float *rho,
                           float *u, float *theta, cudaStream_t s);
