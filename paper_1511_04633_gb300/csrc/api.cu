@@ -42,6 +42,8 @@ struct dmrt {
     bool inplace = false;                 // one buffer, in-place streaming (buf[0])
     int parity = 0;                       // in-place: layout of the state (steps mod 2)
     lbm::InplaceGeometry SI{};
+    bool ab_inplace = false;              // two buffers, plain steps in place by twos
+    lbm::InplaceGeometry ab_SI{};         // and their tables
     long long device_bytes = 0;           // device memory held by the handle
     float *snap = nullptr;                // residual snapshot: theta, u (4 planes)
     double *partials = nullptr;           // reduction scratch (Nu rows; residual block partials)
@@ -180,9 +182,34 @@ cudaError_t launch_one_step(dmrt_t *h, int ph, bool res)
                                        reinterpret_cast<unsigned *>(h->dres + 7), h->K, h->dres, h->stream);
 }
 
-// Does the step from the current step count take a residual point?  The
-// points are the states pulled by the last step of every K-step interval.
-bool residual_step(const dmrt_t *h, long steps_done) { return (steps_done + 1) % h->K == 0; }
+// Two plain steps of a two-buffer state in place, on its own buffer.
+cudaError_t launch_two_steps(dmrt_t *h, int ph)
+{
+    for (int phase : {0, 2}) {
+        const cudaError_t e =
+            h->split ? lbm::launch_step_inplace_split(h->wall, h->storage, h->stochastic, h->buf[ph], phase, h->ab_SI,
+                                                      h->G, h->C, h->stream, h->use_pdl)
+                     : lbm::launch_step_inplace_pair(h->wall, h->storage, h->stochastic, h->buf[ph], phase, h->ab_SI,
+                                                     h->G, h->C, h->stream, h->use_pdl);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// The next step or two from state `ph` (which follows), of which the last may
+// come `until_res` steps from now, when a residual point is due; at most
+// `most`.  *done: the steps launched.
+cudaError_t launch_steps(dmrt_t *h, int &ph, long until_res, long most, long *done)
+{
+    if (h->ab_inplace && most >= 2 && until_res > 2) {
+        *done = 2;
+        return launch_two_steps(h, ph);
+    }
+    *done = 1;
+    const cudaError_t e = launch_one_step(h, ph, until_res == 1);
+    ph ^= 1;
+    return e;
+}
 
 // Forget the residual history (a new state was written).
 dmrt_status reset_residual(dmrt_t *h)
@@ -265,10 +292,7 @@ bool capture_interval(dmrt_t *h, int start)
     }
     int ph = start;
     bool ok = true;
-    for (long s = 0; s < h->K && ok; ++s) {
-        ok = launch_one_step(h, ph, s == h->K - 1) == cudaSuccess;
-        ph ^= 1;
-    }
+    for (long s = 0, m = 0; s < h->K && ok; s += m) ok = launch_steps(h, ph, h->K - s, h->K - s, &m) == cudaSuccess;
     cudaGraph_t graph = nullptr;
     ok = (cudaStreamEndCapture(h->stream, &graph) == cudaSuccess) && ok && graph;
     cudaGraphExec_t exec = nullptr;
@@ -304,6 +328,7 @@ dmrt_status run_steps(dmrt_t *h, long n)
             if (!h->interval_graph[ph] && !capture_interval(h, ph)) h->use_graphs = false;
             if (h->interval_graph[ph]) {
                 CK(h, cudaGraphLaunch(h->interval_graph[ph], h->stream), "cudaGraphLaunch");
+                // (steps taken in place by twos keep the buffer and the parity)
                 if (h->K & 1) ph ^= 1;
                 h->steps += chunk;
                 h->step_launches += chunk;
@@ -312,14 +337,16 @@ dmrt_status run_steps(dmrt_t *h, long n)
                 graphed = true;
             }
         }
-        for (long s = 0; s < chunk && !graphed; ++s) {
-            const bool res = residual_step(h, h->steps);
-            CK(h, launch_one_step(h, ph, res), "step kernel");
-            ph ^= 1;
-            h->steps++;
-            h->step_launches++;
-            h->total_launches += res ? 2 : 1;
-            if (res && h->snaps < 2) h->snaps++;
+        for (long s = 0, m = 0; s < chunk && !graphed; s += m) {
+            const long to_go = h->K - h->steps % h->K;
+            CK(h, launch_steps(h, ph, to_go, chunk - s, &m), "step kernel");
+            h->steps += m;
+            h->step_launches += m;
+            h->total_launches += m;
+            if (to_go == 1) {
+                h->total_launches++;  // the residual's finishing kernel
+                if (h->snaps < 2) h->snaps++;
+            }
         }
         if (h->timing) {
             CK(h, cudaEventRecord(e1, h->stream), "cudaEventRecord");
@@ -423,6 +450,9 @@ dmrt_status create_common(dmrt_t **out, const int grid[3], double nu, double alp
         return DMRT_ERR_ARG;
     }
     h->pair_loads = h->cells_per_thread != 2 || h->inplace ? 0 : (tma_ok && ploads == 2 ? 2 : 1);
+    h->ab_inplace = !h->inplace && ((h->cells_per_thread == 2 && h->pair_loads == 1) || h->split) &&
+                    lbm::inplace_pays(h->G, storage, h->split);
+    if (h->ab_inplace) lbm::fill_ab_inplace_geometry(h->G, h->ab_SI);
 #ifdef DMRT_BLOCK_X
     h->block = {DMRT_BLOCK_X, DMRT_BLOCK_Y};
 #else

@@ -34,6 +34,34 @@ cudaError_t launch_step(int wall, int storage, bool stochastic, const void *src,
                         const StepGeometry &S, const Geometry &G, const CollideParams &C,
                         BlockShape b, cudaStream_t s, bool pdl, const ResidualArgs *res = nullptr);
 
+// Division of numbers n < 2^28 by d: (n * mul) >> shift with shift = 28 +
+// ceil(log2 d) and mul = floor(2^shift / d) + 1.  mul * d exceeds 2^shift by
+// at most d, and n * d < 2^28 * 2^ceil(log2 d), so the quotient is exact.
+struct RowDivisor {
+    unsigned long long mul;
+    unsigned shift;
+    explicit RowDivisor(unsigned d)
+    {
+        unsigned s = 0;
+        while ((1ull << s) < d) ++s;
+        shift = 28 + s;
+        mul = (1ull << shift) / d + 1ull;
+    }
+    __host__ __device__ unsigned divide(unsigned n) const
+    {
+        return static_cast<unsigned>((n * mul) >> shift);
+    }
+};
+
+// Divisors of a box's flat cell index: by a slab's cells and by a row's.
+struct BoxDivisors {
+    RowDivisor row, slab;
+    explicit BoxDivisors(const Geometry &G)
+        : row(static_cast<unsigned>(G.nx)), slab(static_cast<unsigned>(G.nx) * static_cast<unsigned>(G.ny))
+    {
+    }
+};
+
 // The same step with two neighbouring cells of a row per thread (x0 even):
 // bitwise the values of launch_step, in packed FP32x2 arithmetic.  Needs a
 // walled box (wall 1..3) and an even nx (step_pair_supported); the launcher
@@ -42,7 +70,7 @@ bool step_pair_supported(int wall, const Geometry &G);
 cudaError_t launch_step_pair(int wall, int storage, bool stochastic, const void *src, void *dst,
                              const StepGeometry &S, const Geometry &G, const CollideParams &C,
                              cudaStream_t s, bool pdl, const ResidualArgs *res = nullptr);
-// Blocks of the paired kernels' grid (the residual partials they write).
+// Blocks of a paired kernel that takes a residual point (the partials it writes).
 size_t pair_blocks(const Geometry &G);
 
 // In-place streaming (one buffer).  The state alternates between two
@@ -74,29 +102,17 @@ cudaError_t launch_step_pair_tma(int wall, int storage, bool stochastic, const v
 
 // Both in-place phases with two cells per thread (same conditions as
 // launch_step_pair); bitwise the values of launch_step_inplace.
+// A two-buffer cavity can take steps in place too, two at a time on the
+// buffer of its state: phase 0 with the tables of fill_ab_inplace_geometry,
+// then phase 2 (no residual point), which leaves the two-buffer layout and
+// the step counter in the buffer's first counter word again.
+// inplace_pays: is that faster than stepping between the buffers?
+void fill_ab_inplace_geometry(const Geometry &G, InplaceGeometry &SI);
+bool inplace_pays(const Geometry &G, int storage, bool split);
 cudaError_t launch_step_inplace_pair(int wall, int storage, bool stochastic, void *buf, int phase,
                                      const InplaceGeometry &SI, const Geometry &G,
                                      const CollideParams &C, cudaStream_t s, bool pdl,
                                      const ResidualArgs *res = nullptr);
-
-// Division of numbers n < 2^28 by d: (n * mul) >> shift with shift = 28 +
-// ceil(log2 d) and mul = floor(2^shift / d) + 1.  mul * d exceeds 2^shift by
-// at most d, and n * d < 2^28 * 2^ceil(log2 d), so the quotient is exact.
-struct RowDivisor {
-    unsigned long long mul;
-    unsigned shift;
-    explicit RowDivisor(unsigned d)
-    {
-        unsigned s = 0;
-        while ((1ull << s) < d) ++s;
-        shift = 28 + s;
-        mul = (1ull << shift) / d + 1ull;
-    }
-    __host__ __device__ unsigned divide(unsigned n) const
-    {
-        return static_cast<unsigned>((n * mul) >> shift);
-    }
-};
 
 // The same steps for boxes with odd rows, two cells of neighbouring slabs per
 // thread: bitwise the values of launch_step and launch_step_inplace.  Needs

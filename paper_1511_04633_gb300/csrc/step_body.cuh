@@ -461,6 +461,17 @@ struct LocalOffsets {
     __device__ __forceinline__ unsigned bb() const { return Q * plane; }
 };
 
+// The same where phase 0 started from the two-buffer layout: population q
+// arrives in the cell's slot of plane opp(q).
+struct LocalOppOffsets {
+    unsigned plane;
+    static constexpr bool kLocal = true;
+    template <int Q>
+    __device__ __forceinline__ unsigned nb() const { return plane_opp<Q>() * plane; }
+    template <int Q>
+    __device__ __forceinline__ unsigned bb() const { return plane_opp<Q>() * plane; }
+};
+
 // Phase-0 offsets of the in-place scheme computed from the strides: S_q(x -
 // e_q) sits in plane opp(q) at x - e_q (nb), the bounce-back source S_opp(x)
 // in plane q at x (bb); the value leaving x along q goes to plane q at x +

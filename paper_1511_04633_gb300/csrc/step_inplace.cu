@@ -173,6 +173,36 @@ void fill_inplace_geometry(const Geometry &G, InplaceGeometry &SI)
     }
 }
 
+void fill_ab_inplace_geometry(const Geometry &G, InplaceGeometry &SI)
+{
+    // S_q(x) starts in plane q at x: every plane has its opposite's name
+    fill_step_geometry(G, SI.load);
+    const long long sy = G.nx, sz = static_cast<long long>(G.nx) * G.ny;
+    for (int q = 0; q < kPlanes; ++q) {
+        const int ex = q < 19 ? q19_ex(q) : q7_ex(q - 19);
+        const int ey = q < 19 ? q19_ey(q) : q7_ey(q - 19);
+        const int ez = q < 19 ? q19_ez(q) : q7_ez(q - 19);
+        const int opp = q < 19 ? q19_opp(q) : 19 + q7_opp(q - 19);
+        const long long off = ex + ey * sy + ez * sz;
+        SI.sn[q] = static_cast<int>(static_cast<unsigned>(opp * G.plane + off));
+        SI.sb[q] = static_cast<int>(static_cast<unsigned>(q * G.plane));
+    }
+}
+
+// In place, the state is one buffer instead of two: a cavity whose one buffer
+// stays in L2 (129 MB) while two do not steps faster.  Measured on GB300, per
+// step, two buffers -> in place: FP32 80^3 13.3 -> 10.8 us, 96^3 28.2 ->
+// 21.5; 16-bit 96^3 15.7 -> 15.2, 112^3 28.4 -> 23.4, 190 x 126 x 90 41.6 ->
+// 36.7, 128^3 39.5 -> 39.0; below and above (FP32 60^3 5.8 -> 6.1, 112^3 44.1
+// -> 44.9, BF16 142^3 54.6 -> 55.3) two buffers are as fast or faster.  With
+// odd rows (split) the stores between buffers share sectors at every row end
+// and in place stays faster: 127^3 BF16 47.3 -> 42.0, 255^3 375 -> 357 us.
+bool inplace_pays(const Geometry &G, int storage, bool split)
+{
+    const long long bytes = static_cast<long long>(G.plane) * kPlanes * storage_bytes(storage);
+    return 2 * bytes >= 90000000ll && (split || bytes <= 117000000ll);
+}
+
 cudaError_t launch_step_inplace(int wall, int storage, bool stochastic, void *buf, int phase,
                                 const InplaceGeometry &SI, const Geometry &G,
                                 const CollideParams &C, BlockShape b, cudaStream_t s, bool pdl,

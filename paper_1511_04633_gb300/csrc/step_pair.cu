@@ -46,7 +46,6 @@ constexpr int kPairBlocks = DMRT_PAIR_MIN_BLOCKS;
 constexpr int kPairBlocks = 5;
 #endif
 
-// Thread -> pair: x0 = 2 (block x * block width + thread x) must be < nx.
 struct PairCoords {
     int x0, y, z;
     unsigned self;
@@ -55,14 +54,33 @@ struct PairCoords {
     bool valid;
 };
 
-__device__ __forceinline__ PairCoords pair_coords(const StepGeometry &S)
+// Thread -> pair.
+// FLAT: the pairs of the whole box are numbered in memory order, so a
+// block's accesses are runs of consecutive cells and no lane idles at the
+// end of a row or slab, whatever the row length; the coordinates take two
+// multiplications (BoxDivisors).
+// Otherwise a block is blockDim.x pairs of a row by blockDim.y rows of the
+// slab blockIdx.z, and the z faces are the same for the whole block.
+template <bool FLAT>
+__device__ __forceinline__ PairCoords pair_coords(const StepGeometry &S, const BoxDivisors &D)
 {
     PairCoords c;
-    c.x0 = 2 * static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
-    c.y = blockIdx.y * blockDim.y + threadIdx.y;
-    c.z = blockIdx.z;
-    c.valid = c.x0 < S.nx && c.y < S.ny;
-    c.self = (static_cast<unsigned>(c.z) * S.ny + c.y) * S.nx + c.x0;
+    if constexpr (FLAT) {
+        c.self = 2u * (blockIdx.x * blockDim.x + threadIdx.x);
+        const unsigned nx = static_cast<unsigned>(S.nx), nxy = nx * S.ny;
+        c.valid = c.self < nxy * S.nz;
+        const unsigned z = D.slab.divide(c.self), r = c.self - z * nxy;
+        const unsigned y = D.row.divide(r);
+        c.x0 = static_cast<int>(r - y * nx);
+        c.y = static_cast<int>(y);
+        c.z = static_cast<int>(z);
+    } else {
+        c.x0 = 2 * static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+        c.y = blockIdx.y * blockDim.y + threadIdx.y;
+        c.z = blockIdx.z;
+        c.valid = c.x0 < S.nx && c.y < S.ny;
+        c.self = (static_cast<unsigned>(c.z) * S.ny + c.y) * S.nx + c.x0;
+    }
     c.faces = {c.x0 == 0, c.x0 + 2 == S.nx, c.y == 0, c.y == S.ny - 1, c.z == 0, c.z == S.nz - 1};
     c.th_lin = theta_linear(c.y, S.inv_ny);
     return c;
@@ -85,15 +103,18 @@ constexpr int kPairBlocksRes = 4;
 
 // RES: this step also takes a residual point of the state it pulls (the
 // fields of the pulled populations against the snapshot, residual.cuh).
-template <int WALL, typename T, bool SR, bool RES>
+// The divisors come last among the parameters: ahead of C they moved it to
+// an 8-byte boundary, the compiler then fetched its constants in pairs into
+// registers, and the BF16 step took 8 % longer (256^3: 318 against 294 us).
+template <int WALL, typename T, bool SR, bool RES, bool FLAT>
 __global__ void __launch_bounds__(kPairThreads, RES ? kPairBlocksRes : kPairBlocks)
     step_pair_kernel(const T *__restrict__ src, T *__restrict__ dst, const StepGeometry S,
-                     const CollideParams C, const ResidualArgs R)
+                     const CollideParams C, const ResidualArgs R, const BoxDivisors D)
 {
     // programmatic dependent launch, as in the one-cell kernel
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    const PairCoords c = pair_coords(S);
+    const PairCoords c = pair_coords<FLAT>(S, D);
     DF acc[4] = {};
     if (c.valid) {
         F2 d[19], g[7];
@@ -128,29 +149,33 @@ __global__ void __launch_bounds__(kPairThreads, RES ? kPairBlocksRes : kPairBloc
 // pair; phase 0 pulls like the two-buffer step and writes S*_q to x + e_q,
 // an aligned pair for the planes with e_x = 0 and one element per cell for
 // the others (or, where the link leaves the box, plane opp(q) at the cell).
-template <int WALL, typename T, bool SR, int PHASE, bool RES>
+// PHASE 2 is phase 1 for a buffer that started in the two-buffer layout: the
+// planes have their opposites' names (fill_ab_inplace_geometry gives phase 0
+// the matching tables).
+template <int WALL, typename T, bool SR, int PHASE, bool RES, bool FLAT>
 __global__ void __launch_bounds__(kPairThreads, RES ? kPairBlocksRes : kPairBlocks)
     step_inplace_pair_kernel(T *__restrict__ A, const InplaceGeometry SI, const CollideParams C,
-                             const ResidualArgs R)
+                             const ResidualArgs R, const BoxDivisors D)
 {
     const StepGeometry &S = SI.load;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    const PairCoords c = pair_coords(S);
+    const PairCoords c = pair_coords<FLAT>(S, D);
     DF acc[4] = {};
     if (c.valid) {
         F2 d[19], g[7];
         float2 prev[4];
         if constexpr (RES) residual_pair_load(R, c.self, prev);
         if constexpr (PHASE == 0) pull_pair<WALL, T>(A + c.self, TableOffsets{S}, c.faces, c.th_lin, d, g);
-        else pull_pair<WALL, T>(A + c.self, LocalOffsets{S.plane}, c.faces, c.th_lin, d, g);
+        else if constexpr (PHASE == 1) pull_pair<WALL, T>(A + c.self, LocalOffsets{S.plane}, c.faces, c.th_lin, d, g);
+        else pull_pair<WALL, T>(A + c.self, LocalOppOffsets{S.plane}, c.faces, c.th_lin, d, g);
         const Conserved<F2> m0 = conserved<F2, Pair<T>::kShift>(d, g);
         const PairFields fl{m0.Tu, m0.vx, m0.vy, m0.vz};
         unsigned r01 = 0;
         if constexpr (SR) {
             unsigned *ctr = reinterpret_cast<unsigned *>(A + static_cast<size_t>(kPlanes) * S.plane);
-            const unsigned step = ctr[PHASE];
-            if (c.self == 0) ctr[PHASE ^ 1] = step + 1u;
+            const unsigned step = ctr[PHASE != 0];
+            if (c.self == 0) ctr[PHASE == 0] = step + 1u;
             r01 = pair_bits(c.self, step);
         }
         T *Dp = A + c.self;
@@ -161,6 +186,8 @@ __global__ void __launch_bounds__(kPairThreads, RES ? kPairBlocksRes : kPairBloc
             const unsigned r = SR ? plane_bits<q>(r01) : 0u;
             if constexpr (PHASE == 1) {
                 store2<T, SR>(Dp + plane_opp<q>() * plane, v, r);
+            } else if constexpr (PHASE == 2) {
+                store2<T, SR>(Dp + q * plane, v, r);
             } else {
                 constexpr int ex = plane_ex<q>(), ey = plane_ey<q>(), ez = plane_ez<q>();
                 bool lyz = false;  // the link leaves through a y or z face
@@ -416,24 +443,64 @@ bool step_pair_supported(int wall, const Geometry &G)
 
 namespace {
 
-// Launch shape of the paired kernels: one row of up to 128 cells per block
-// row, kPairThreads threads per block.
-cudaLaunchConfig_t pair_config(const Geometry &G, cudaStream_t s, cudaLaunchAttribute *attr, bool pdl)
+// The block tile of a row-wise launch: the width (in pairs) that leaves the
+// fewest idle threads along a row, the widest of equals (48 pairs take 3
+// tiles of 16, not 2 of 32).
+int tile_width(int row, int &slots)
 {
-    const int threads = kPairThreads;
-    const int pairs = G.nx / 2;
-    // the tile width (in pairs) that launches the fewest idle threads along a
-    // row, the widest of equals: 48 pairs take 3 tiles of 16, not 2 of 32
-    int bx = 16, slots = (pairs + 15) / 16 * 16;
+    int bx = 16;
+    slots = (row + 15) / 16 * 16;
     for (int cand : {32, 64}) {
-        const int c = (pairs + cand - 1) / cand * cand;
+        const int c = (row + cand - 1) / cand * cand;
         if (c <= slots) bx = cand, slots = c;
     }
-    const int by = threads / bx > 0 ? threads / bx : 1;
+    return bx;
+}
+
+// Flat numbering of the pairs, or row tiles?  Flat costs the collision's 16-
+// bit step 2 to 4 % (the coordinates, and z faces that differ within a
+// block), and gains where row tiles idle lanes or, with two buffers, where
+// rows are not whole 64-byte lines, so that the tiles' stores share sectors.
+// Measured on GB300, per step, row tiles -> flat:
+//   two buffers  FP32 12 x 250 x 250 36.3 -> 23.7 us, 70^3 11.5 -> 7.7, 130^3
+//     90 -> 68, 222^3 402 -> 327; BF16 12 x 250 x 250 31.3 -> 13.1, 130^3
+//     54.7 -> 42.6, 190 x 126 x 90 44.3 -> 41.6; but 256^3 293.6 -> 300.3
+//   in place     BF16 70^3 9.7 -> 7.3, 112^3 26.0 -> 23.4; but 190 x 126 x 90
+//     (1 % idle) 36.7 -> 40.2, FP32 60^3 (6 %) 6.08 -> 6.22
+// Boxes of 2.5 to 4 flat blocks per SM keep the tiles: FP32 48^3 4.5 -> 5.0
+// us, 52^3 4.7 -> 4.9; so do the smallest in place (16^3: 1.94 -> 2.07).
+// A step that takes a residual point always uses the row tiles: the order of
+// its sums, and so the residual, is then the same in either scheme.
+bool pair_flat(const Geometry &G, bool inplace, bool res)
+{
+    if (res) return false;
+    int slots;
+    const int row = G.nx / 2, bx = tile_width(row, slots), by = kPairThreads / bx;
+    const long long pairs = static_cast<long long>(row) * G.ny * G.nz;
+    const long long blocks = (pairs + kPairThreads - 1) / kPairThreads;
+    if ((blocks > 380 && blocks <= 610) || (inplace && blocks <= 100)) return false;
+    const double idle = 1.0 - static_cast<double>(row) * G.ny / (static_cast<double>(slots) * ((G.ny + by - 1) / by * by));
+    return inplace ? idle > 0.08 : idle > 0.03 || G.nx % 32 != 0;
+}
+
+// Launch shape of the paired kernels (pair_coords).
+cudaLaunchConfig_t pair_config(const Geometry &G, bool inplace, bool res, cudaStream_t s, cudaLaunchAttribute *attr,
+                               bool pdl)
+{
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((pairs + bx - 1) / bx, (G.ny + by - 1) / by, G.nz);
-    cfg.blockDim = dim3(bx, by, 1);
-    cfg.dynamicSmemBytes = 0;
+    if (pair_flat(G, inplace, res)) {
+        const long long pairs = static_cast<long long>(G.nx / 2) * G.ny * G.nz;
+        // up to two blocks per SM: half as large ones spread further (36^3
+        // FP32 2.9 -> 2.6 us)
+        const int threads = pairs <= 2 * 152 * kPairThreads ? kPairThreads / 2 : kPairThreads;
+        cfg.gridDim = dim3(static_cast<unsigned>((pairs + threads - 1) / threads));
+        cfg.blockDim = dim3(threads);
+    } else {
+        int slots;
+        const int row = G.nx / 2, bx = tile_width(row, slots), by = kPairThreads / bx;
+        cfg.gridDim = dim3((row + bx - 1) / bx, (G.ny + by - 1) / by, G.nz);
+        cfg.blockDim = dim3(bx, by, 1);
+    }
     cfg.stream = s;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -447,7 +514,7 @@ cudaLaunchConfig_t pair_config(const Geometry &G, cudaStream_t s, cudaLaunchAttr
 size_t pair_blocks(const Geometry &G)
 {
     cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = pair_config(G, nullptr, attr, false);
+    const cudaLaunchConfig_t cfg = pair_config(G, false, true, nullptr, attr, false);
     return static_cast<size_t>(cfg.gridDim.x) * cfg.gridDim.y * cfg.gridDim.z;
 }
 
@@ -457,8 +524,9 @@ cudaError_t launch_step_pair(int wall, int storage, bool stochastic, const void 
 {
     if (!step_pair_supported(wall, G)) return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pair_config(G, s, attr, pdl);
+    cudaLaunchConfig_t cfg = pair_config(G, false, res != nullptr, s, attr, pdl);
     const ResidualArgs R = res ? *res : ResidualArgs{};
+    const BoxDivisors D(G);
     cudaError_t e = dispatch(wall, storage, [&](auto W, auto *tp) {
         using T = std::remove_pointer_t<decltype(tp)>;
         constexpr int WL = decltype(W)::value;
@@ -467,15 +535,16 @@ cudaError_t launch_step_pair(int wall, int storage, bool stochastic, const void 
         } else {
             const T *a = static_cast<const T *>(src);
             T *b = static_cast<T *>(dst);
-            auto go = [&](auto sr) {
-                constexpr bool SRv = decltype(sr)::value;
-                if (res) return cudaLaunchKernelEx(&cfg, step_pair_kernel<WL, T, SRv, true>, a, b, S, C, R);
-                return cudaLaunchKernelEx(&cfg, step_pair_kernel<WL, T, SRv, false>, a, b, S, C, R);
+            auto go = [&](auto sr, auto flat) {
+                constexpr bool SRv = decltype(sr)::value, FL = decltype(flat)::value;
+                if (res) return cudaLaunchKernelEx(&cfg, step_pair_kernel<WL, T, SRv, true, false>, a, b, S, C, R, D);
+                return cudaLaunchKernelEx(&cfg, step_pair_kernel<WL, T, SRv, false, FL>, a, b, S, C, R, D);
             };
+            auto by_shape = [&](auto sr) { return pair_flat(G, false, res != nullptr) ? go(sr, std::true_type{}) : go(sr, std::false_type{}); };
             if constexpr (!std::is_same_v<T, float>) {
-                if (stochastic) return go(std::true_type{});
+                if (stochastic) return by_shape(std::true_type{});
             }
-            return go(std::false_type{});
+            return by_shape(std::false_type{});
         }
     });
     if (e != cudaSuccess) return e;
@@ -583,10 +652,11 @@ cudaError_t launch_step_inplace_pair(int wall, int storage, bool stochastic, voi
                                      const CollideParams &C, cudaStream_t s, bool pdl,
                                      const ResidualArgs *res)
 {
-    if (!step_pair_supported(wall, G) || (phase != 0 && phase != 1)) return cudaErrorInvalidValue;
+    if (!step_pair_supported(wall, G) || phase < 0 || phase > 2 || (phase == 2 && res)) return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pair_config(G, s, attr, pdl);
+    cudaLaunchConfig_t cfg = pair_config(G, true, res != nullptr, s, attr, pdl);
     const ResidualArgs R = res ? *res : ResidualArgs{};
+    const BoxDivisors D(G);
     cudaError_t e = dispatch(wall, storage, [&](auto W, auto *tp) {
         using T = std::remove_pointer_t<decltype(tp)>;
         constexpr int WL = decltype(W)::value;
@@ -594,20 +664,26 @@ cudaError_t launch_step_inplace_pair(int wall, int storage, bool stochastic, voi
             return cudaErrorInvalidValue;
         } else {
             T *A = static_cast<T *>(buf);
-            auto go = [&](auto sr) {
-                constexpr bool SRv = decltype(sr)::value;
+            auto go = [&](auto sr, auto flat) {
+                constexpr bool SRv = decltype(sr)::value, FL = decltype(flat)::value;
+                auto run = [&](auto ph, auto rs) {
+                    constexpr bool RS = decltype(rs)::value;
+                    return cudaLaunchKernelEx(&cfg, step_inplace_pair_kernel<WL, T, SRv, decltype(ph)::value, RS, FL && !RS>,
+                                              A, SI, C, R, D);
+                };
+                using std::integral_constant;
+                if (phase == 2) return run(integral_constant<int, 2>{}, std::false_type{});
                 if (res)
-                    return phase == 0
-                               ? cudaLaunchKernelEx(&cfg, step_inplace_pair_kernel<WL, T, SRv, 0, true>, A, SI, C, R)
-                               : cudaLaunchKernelEx(&cfg, step_inplace_pair_kernel<WL, T, SRv, 1, true>, A, SI, C, R);
-                return phase == 0
-                           ? cudaLaunchKernelEx(&cfg, step_inplace_pair_kernel<WL, T, SRv, 0, false>, A, SI, C, R)
-                           : cudaLaunchKernelEx(&cfg, step_inplace_pair_kernel<WL, T, SRv, 1, false>, A, SI, C, R);
+                    return phase == 0 ? run(integral_constant<int, 0>{}, std::true_type{})
+                                      : run(integral_constant<int, 1>{}, std::true_type{});
+                return phase == 0 ? run(integral_constant<int, 0>{}, std::false_type{})
+                                  : run(integral_constant<int, 1>{}, std::false_type{});
             };
+            auto by_shape = [&](auto sr) { return pair_flat(G, true, res != nullptr) ? go(sr, std::true_type{}) : go(sr, std::false_type{}); };
             if constexpr (!std::is_same_v<T, float>) {
-                if (stochastic) return go(std::true_type{});
+                if (stochastic) return by_shape(std::true_type{});
             }
-            return go(std::false_type{});
+            return by_shape(std::false_type{});
         }
     });
     if (e != cudaSuccess) return e;

@@ -151,8 +151,8 @@ __device__ __forceinline__ void residual_split(const ResidualArgs &R, const Spli
 
 template <int WALL, typename T, bool SR, bool RES>
 __global__ void __launch_bounds__(kSplitThreads, RES ? kSplitBlocksRes : kSplitBlocks)
-    step_split_kernel(const T *__restrict__ src, T *__restrict__ dst, const StepGeometry S, const RowDivisor D,
-                      const CollideParams C, const ResidualArgs R)
+    step_split_kernel(const T *__restrict__ src, T *__restrict__ dst, const StepGeometry S,
+                      const CollideParams C, const ResidualArgs R, const RowDivisor D)
 {
     // programmatic dependent launch, as in the one-cell kernel
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -187,11 +187,11 @@ __global__ void __launch_bounds__(kSplitThreads, RES ? kSplitBlocksRes : kSplitB
     if constexpr (RES) residual_block_store(acc, R.partials);
 }
 
-// The two in-place phases (step_inplace.cu).
+// The two in-place phases (step_inplace.cu); PHASE 2 as in step_pair.cu.
 template <int WALL, typename T, bool SR, int PHASE, bool RES>
 __global__ void __launch_bounds__(kSplitThreads, RES ? kSplitBlocksRes : kSplitBlocks)
-    step_inplace_split_kernel(T *__restrict__ A, const InplaceGeometry SI, const RowDivisor D, const CollideParams C,
-                              const ResidualArgs R)
+    step_inplace_split_kernel(T *__restrict__ A, const InplaceGeometry SI, const CollideParams C,
+                              const ResidualArgs R, const RowDivisor D)
 {
     const StepGeometry &S = SI.load;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -206,14 +206,15 @@ __global__ void __launch_bounds__(kSplitThreads, RES ? kSplitBlocksRes : kSplitB
             residual_cell_load(R, p.c1, p1);
         }
         if constexpr (PHASE == 0) pull_split<WALL, T>(A + p.c0, A + p.c1, TableOffsets{S}, p, d, g);
-        else pull_split<WALL, T>(A + p.c0, A + p.c1, LocalOffsets{S.plane}, p, d, g);
+        else if constexpr (PHASE == 1) pull_split<WALL, T>(A + p.c0, A + p.c1, LocalOffsets{S.plane}, p, d, g);
+        else pull_split<WALL, T>(A + p.c0, A + p.c1, LocalOppOffsets{S.plane}, p, d, g);
         const Conserved<F2> m0 = conserved<F2, Pair<T>::kShift>(d, g);
         const float2 th = m0.Tu.v, ux = m0.vx.v, uy = m0.vy.v, uz = m0.vz.v;
         unsigned r01 = 0;
         if constexpr (SR) {
             unsigned *ctr = reinterpret_cast<unsigned *>(A + static_cast<size_t>(kPlanes) * S.plane);
-            const unsigned step = ctr[PHASE];
-            if (p.c0 == 0) ctr[PHASE ^ 1] = step + 1u;
+            const unsigned step = ctr[PHASE != 0];
+            if (p.c0 == 0) ctr[PHASE == 0] = step + 1u;
             r01 = split_bits(p, step);
         }
         T *D0 = A + p.c0, *D1 = A + p.c1;
@@ -223,6 +224,8 @@ __global__ void __launch_bounds__(kSplitThreads, RES ? kSplitBlocksRes : kSplitB
             const unsigned r = SR ? plane_bits<q>(r01) : 0u;
             if constexpr (PHASE == 1) {
                 store_both<T, SR>(D0 + plane_opp<q>() * plane, D1 + plane_opp<q>() * plane, p.two, v, r);
+            } else if constexpr (PHASE == 2) {
+                store_both<T, SR>(D0 + q * plane, D1 + q * plane, p.two, v, r);
             } else {
                 bool l0, l1;  // the link leaves the box
                 split_outside<q, false>(p, l0, l1);
@@ -302,8 +305,8 @@ cudaError_t launch_step_split(int wall, int storage, bool stochastic, const void
         constexpr bool SRv = decltype(sr)::value;
         const T *a = static_cast<const T *>(src);
         T *b = static_cast<T *>(dst);
-        return res ? cudaLaunchKernelEx(&cfg, step_split_kernel<WL, T, SRv, true>, a, b, S, D, C, R)
-                   : cudaLaunchKernelEx(&cfg, step_split_kernel<WL, T, SRv, false>, a, b, S, D, C, R);
+        return res ? cudaLaunchKernelEx(&cfg, step_split_kernel<WL, T, SRv, true>, a, b, S, C, R, D)
+                   : cudaLaunchKernelEx(&cfg, step_split_kernel<WL, T, SRv, false>, a, b, S, C, R, D);
     });
 }
 
@@ -311,7 +314,7 @@ cudaError_t launch_step_inplace_split(int wall, int storage, bool stochastic, vo
                                       const InplaceGeometry &SI, const Geometry &G, const CollideParams &C,
                                       cudaStream_t s, bool pdl, const ResidualArgs *res)
 {
-    if (!step_split_supported(wall, G) || (phase != 0 && phase != 1)) return cudaErrorInvalidValue;
+    if (!step_split_supported(wall, G) || phase < 0 || phase > 2 || (phase == 2 && res)) return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = split_config(G, s, attr, pdl);
     const ResidualArgs R = res ? *res : ResidualArgs{};
@@ -321,11 +324,17 @@ cudaError_t launch_step_inplace_split(int wall, int storage, bool stochastic, vo
         constexpr int WL = decltype(W)::value;
         constexpr bool SRv = decltype(sr)::value;
         T *A = static_cast<T *>(buf);
+        auto run = [&](auto ph, auto rs) {
+            return cudaLaunchKernelEx(
+                &cfg, step_inplace_split_kernel<WL, T, SRv, decltype(ph)::value, decltype(rs)::value>, A, SI, C, R, D);
+        };
+        using std::integral_constant;
+        if (phase == 2) return run(integral_constant<int, 2>{}, std::false_type{});
         if (res)
-            return phase == 0 ? cudaLaunchKernelEx(&cfg, step_inplace_split_kernel<WL, T, SRv, 0, true>, A, SI, D, C, R)
-                              : cudaLaunchKernelEx(&cfg, step_inplace_split_kernel<WL, T, SRv, 1, true>, A, SI, D, C, R);
-        return phase == 0 ? cudaLaunchKernelEx(&cfg, step_inplace_split_kernel<WL, T, SRv, 0, false>, A, SI, D, C, R)
-                          : cudaLaunchKernelEx(&cfg, step_inplace_split_kernel<WL, T, SRv, 1, false>, A, SI, D, C, R);
+            return phase == 0 ? run(integral_constant<int, 0>{}, std::true_type{})
+                              : run(integral_constant<int, 1>{}, std::true_type{});
+        return phase == 0 ? run(integral_constant<int, 0>{}, std::false_type{})
+                          : run(integral_constant<int, 1>{}, std::false_type{});
     });
 }
 

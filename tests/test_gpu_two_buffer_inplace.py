@@ -1,0 +1,59 @@
+"""Two-buffer cavities of the sizes whose plain steps run in place by twos
+(inplace_pays), and the flat numbering of the paired kernels, against the
+one-cell two-buffer kernels, bitwise."""
+
+import numpy as np
+import pytest
+
+from paper_1511_04633_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dm():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1511_04633_gb300 import dmrt
+    return dmrt
+
+
+def _cavity(dm, grid, wall, storage, cpt, K):
+    cav = dm.Cavity(grid, 1e5, wall_type=wall, storage=storage, cells_per_thread=cpt, residual_interval=K)
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12, np.float32)[:, None, None, None]
+    f = w * (19 * inputs.random_populations(grid, 19, seed=3, spread=0.02))
+    cav.set_populations(f, inputs.random_thermal_populations(grid, seed=4))
+    return cav
+
+
+# the smallest and largest working sets of the rule (433,000 cells FP32, 2.2
+# million 16-bit), row tiles and flat blocks, odd rows; odd and even residual
+# intervals; then boxes outside the rule for the flat numbering: thin, two
+# cells wide, few blocks, a last block with one pair
+@pytest.mark.parametrize("grid,wall,storage,K", [
+    ((130, 96, 48), 2, 0, 6), ((96, 96, 48), 1, 0, 7), ((114, 96, 100), 3, 0, 2), ((190, 80, 60), 3, 1, 5),
+    ((128, 128, 128), 1, 2, 4), ((101, 75, 61), 2, 0, 7), ((129, 90, 80), 3, 1, 6), ((127, 97, 121), 1, 2, 3),
+    ((12, 250, 250), 2, 1, 6), ((2, 300, 129), 1, 0, 5), ((36, 36, 36), 3, 2, 4), ((130, 130, 3), 2, 0, 3),
+])
+def test_bitwise_the_one_cell_kernels(dm, grid, wall, storage, K):
+    a = _cavity(dm, grid, wall, storage, 0, K)
+    b = _cavity(dm, grid, wall, storage, 1, K)
+    for n in (1, 2, 3, 2 * K, K + 3):
+        a.step(n)
+        b.step(n)
+        for p, q in zip(a.populations(), b.populations()):
+            assert np.array_equal(p, q)
+    for p, q in zip(a.fields(), b.fields()):
+        assert np.array_equal(p, q)
+    assert a.nusselt(1) == b.nusselt(1)
+    assert abs(a.residual() - b.residual()) <= 1e-12 * b.residual()
+    # a checkpoint of either continues in the other
+    blob = a.save()
+    b.load(blob)
+    a.step(3)
+    b.step(3)
+    for p, q in zip(a.populations(), b.populations()):
+        assert np.array_equal(p, q)
+    a.close()
+    b.close()
