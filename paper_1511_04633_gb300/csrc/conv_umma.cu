@@ -184,6 +184,8 @@ __global__ void __launch_bounds__(kThreads, KG == 2 ? 4 : 2)
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
+    chain_wait();
+    chain_release();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);  // known to be uniform
     bool ok = true;
     if (warp > kMmaWarp) {
@@ -411,6 +413,8 @@ __global__ void __launch_bounds__(kThreads)
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
+    chain_wait();
+    chain_release();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);  // known to be uniform
     bool ok = true;
     if (warp > kMmaWarp) {
@@ -554,7 +558,7 @@ constexpr unsigned kSmemPerCta = 227u * 1024u, kSmemPerSm = 228u * 1024u;
 
 template <int CO, int KG, typename TO>
 cudaError_t launch_narrow(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
-                          int cin, int act, int *err, cudaStream_t s)
+                          int cin, int act, int *err, cudaStream_t s, bool chained)
 {
     constexpr unsigned smem = narrow_smem<CO, KG>();
     auto kernel = conv3d_umma_narrow_kernel<CO, KG, TO>;
@@ -567,8 +571,8 @@ cudaError_t launch_narrow(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const 
     // (a run loads two planes more than it computes)
     const long long planes = static_cast<long long>(batch) * (n / kX) * (n / kY) * n;
     const long long ctas = std::min<long long>(std::max(1, per_sm) * sm_count(), (planes + kMinRun - 1) / kMinRun);
-    kernel<<<static_cast<unsigned>(ctas), kThreads, smem, s>>>(x, w, bias, y, n, cin, act, planes, err);
-    return cudaGetLastError();
+    return launch_chained(kernel, static_cast<unsigned>(ctas), kThreads, smem, s, chained, x, w, bias, y, n, cin, act,
+                          planes, err);
 }
 
 // A choice of CO, R and stages for the wide kernel and its estimated cycles.
@@ -600,20 +604,20 @@ void consider(WideShape &best, long long tiles, int nz, int cin, int cout)
 
 template <int CO, int R, bool PAIR, typename TO>
 cudaError_t launch_wide(const WideShape &sh, long long tiles, const __nv_bfloat16 *x, const __nv_bfloat16 *w,
-                        const float *bias, TO *y, int n, int cin, int cout, int act, int *err, cudaStream_t s)
+                        const float *bias, TO *y, int n, int cin, int cout, int act, int *err, cudaStream_t s,
+                        bool chained)
 {
     const unsigned smem = kHead + table_bytes<PAIR>(R) + sh.stages * stage_bytes<CO, PAIR>(R);
     auto kernel = conv3d_umma_wide_kernel<CO, R, PAIR, TO>;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    kernel<<<dim3(static_cast<unsigned>(tiles / R), cout / CO), kThreads, smem, s>>>(x, w, bias, y, n, cin, cout, act,
-                                                                                   sh.stages, err);
-    return cudaGetLastError();
+    return launch_chained(kernel, dim3(static_cast<unsigned>(tiles / R), cout / CO), kThreads, smem, s, chained, x, w, bias,
+                          y, n, cin, cout, act, sh.stages, err);
 }
 
 template <bool PAIR, typename TO>
 cudaError_t run_wide(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
-                     int cin, int cout, int act, int *err, cudaStream_t s)
+                     int cin, int cout, int act, int *err, cudaStream_t s, bool chained)
 {
     const int nz = PAIR ? n / 2 : n;
     const long long tiles = static_cast<long long>(batch) * (n / kX) * (n / (PAIR ? 8 : 16)) * nz;
@@ -626,7 +630,7 @@ cudaError_t run_wide(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float
     consider<16, 1, PAIR>(sh, tiles, nz, cin, cout);
     auto go = [&](auto co, auto r) {
         return launch_wide<decltype(co)::value, decltype(r)::value, PAIR, TO>(sh, tiles, x, w, bias, y, n, cin, cout, act,
-                                                                              err, s);
+                                                                              err, s, chained);
     };
     auto by_r = [&](auto co) {
         return sh.R == 4 ? go(co, std::integral_constant<int, 4>{}) : go(co, std::integral_constant<int, 1>{});
@@ -665,24 +669,24 @@ bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, i
 
 template <typename TO>
 cudaError_t conv3d_umma(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
-                        int cin, int cout, int act, cudaStream_t s)
+                        int cin, int cout, int act, cudaStream_t s, bool chained)
 {
     int *err = umma_error_word();
     if (!err) return cudaErrorInvalidValue;
     if (n % kY == 0 && cin <= 32 && (cout == 16 || cout == 32)) {
-        if (cout == 16 && cin <= 16) return launch_narrow<16, 2, TO>(x, w, bias, y, batch, n, cin, act, err, s);
-        if (cout == 16) return launch_narrow<16, 4, TO>(x, w, bias, y, batch, n, cin, act, err, s);
-        if (cin <= 16) return launch_narrow<32, 2, TO>(x, w, bias, y, batch, n, cin, act, err, s);
-        return launch_narrow<32, 4, TO>(x, w, bias, y, batch, n, cin, act, err, s);
+        if (cout == 16 && cin <= 16) return launch_narrow<16, 2, TO>(x, w, bias, y, batch, n, cin, act, err, s, chained);
+        if (cout == 16) return launch_narrow<16, 4, TO>(x, w, bias, y, batch, n, cin, act, err, s, chained);
+        if (cin <= 16) return launch_narrow<32, 2, TO>(x, w, bias, y, batch, n, cin, act, err, s, chained);
+        return launch_narrow<32, 4, TO>(x, w, bias, y, batch, n, cin, act, err, s, chained);
     }
-    if (n % kY == 0) return run_wide<false, TO>(x, w, bias, y, batch, n, cin, cout, act, err, s);
-    return run_wide<true, TO>(x, w, bias, y, batch, n, cin, cout, act, err, s);
+    if (n % kY == 0) return run_wide<false, TO>(x, w, bias, y, batch, n, cin, cout, act, err, s, chained);
+    return run_wide<true, TO>(x, w, bias, y, batch, n, cin, cout, act, err, s, chained);
 }
 
 template cudaError_t conv3d_umma<float>(const __nv_bfloat16 *, const __nv_bfloat16 *, const float *, float *, int, int,
-                                        int, int, int, cudaStream_t);
+                                        int, int, int, cudaStream_t, bool);
 template cudaError_t conv3d_umma<__nv_bfloat16>(const __nv_bfloat16 *, const __nv_bfloat16 *, const float *,
-                                                __nv_bfloat16 *, int, int, int, int, int, cudaStream_t);
+                                                __nv_bfloat16 *, int, int, int, int, int, cudaStream_t, bool);
 
 }  // namespace nn
 }  // namespace lbm

@@ -423,6 +423,8 @@ __global__ void __launch_bounds__(256, 2) wgrad_taps_kernel(const __nv_bfloat16 
                                                             int total_tiles, int tiles_per_block)
 {
     extern __shared__ __align__(16) unsigned char wt_smem[];
+    chain_wait();
+    chain_release();
     typedef __nv_bfloat16 Row[kWtRow];
     const int ci_tiles = cin > 8 ? cin / 16 : 1;
     const int co0 = (blockIdx.x / ci_tiles) * 16, ci0 = (blockIdx.x % ci_tiles) * 16;
@@ -1160,6 +1162,8 @@ __device__ __forceinline__ void stn(T *p, const FN<N> &r)
 template <typename T, int N>
 __global__ void avgpool2_kernel(const T *__restrict__ x, T *__restrict__ y, int batch, int n, int c)
 {
+    chain_wait();
+    chain_release();
     const int m = n / 2, c4 = c / (4 * N);
     const long long len = static_cast<long long>(batch) * m * m * m * c4;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
@@ -1208,6 +1212,8 @@ template <typename T, int N>
 __global__ void up2_add_kernel(const T *__restrict__ x, const T *__restrict__ skip, T *__restrict__ y,
                                int batch, int n, int c)
 {
+    chain_wait();
+    chain_release();
     const int m = 2 * n, c4 = c / (4 * N);
     const long long len = static_cast<long long>(batch) * m * m * m * c4;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < len;
@@ -1338,6 +1344,8 @@ __global__ void features_kernel(const double *__restrict__ ra, const int *__rest
 {
     // the per-sample feature (log10 Ra - 4.5) / 1.5, once per block (FP64 is slow)
     extern __shared__ float feat_ra[];
+    chain_wait();
+    chain_release();
     for (int b = threadIdx.x; b < batch; b += blockDim.x)
         feat_ra[b] = static_cast<float>((log10(ra[b]) - 4.5) / 1.5);
     __syncthreads();
@@ -1467,7 +1475,7 @@ unsigned flat_blocks(long long len)
 
 template <typename TI, typename TW, typename TO>
 cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch, int n, int cin,
-                   int cout, int k, int act, cudaStream_t s)
+                   int cout, int k, int act, cudaStream_t s, bool chained)
 {
     if (n % kTile != 0 || (k != 1 && k != 3)) return cudaErrorInvalidValue;
     if (k == 1 && cin <= 16 && cout <= 16 && (cin < 8 || cout < 8)) {
@@ -1484,7 +1492,7 @@ cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch
         const bool aligned =
             ((reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(w)) & 15ull) == 0;
         if (k == 3 && conv3d_umma_takes(x, w, y, batch, n, cin, cout))
-            return conv3d_umma(x, w, bias, y, batch, n, cin, cout, act, s);
+            return conv3d_umma(x, w, bias, y, batch, n, cin, cout, act, s, chained);
         if (k == 3 && aligned && (cin == 8 || cin % 16 == 0) && cout % 16 == 0 && n % kWtX == 0 &&
             n % kWtZ == 0) {
             const unsigned vtiles = static_cast<unsigned>(batch) * (n / kWtX) * (n / kWtY) * (n / kWtZ);
@@ -1546,9 +1554,8 @@ cudaError_t conv3d_wgrad_partials(const __nv_bfloat16 *x, const __nv_bfloat16 *d
     const cudaError_t e =
         cudaFuncSetAttribute(wgrad_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kWtStage);
     if (e != cudaSuccess) return e;
-    wgrad_taps_kernel<<<grid, 256, 2 * kWtStage, s>>>(x, dy, partials, n, cin, cout, tiles_per_sample, static_cast<int>(tiles),
-                                           static_cast<int>(per));
-    return cudaGetLastError();
+    return launch_chained(wgrad_taps_kernel, grid, 256, 2 * kWtStage, s, true, x, dy, partials, n, cin, cout,
+                          tiles_per_sample, static_cast<int>(tiles), static_cast<int>(per));
 }
 
 cudaError_t conv3d_wgrad_bf16(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *dw, float *scratch,
@@ -1710,10 +1717,8 @@ cudaError_t avgpool2(const T *x, T *y, int batch, int n, int c, cudaStream_t s)
     if (c % 4 != 0) return cudaErrorInvalidValue;
     const long long len = static_cast<long long>(batch) * (n / 2) * (n / 2) * (n / 2) * (c / 4);
     if (std::is_same_v<T, __nv_bfloat16> && c % 8 == 0)
-        avgpool2_kernel<T, 2><<<flat_blocks(len / 2), 256, 0, s>>>(x, y, batch, n, c);
-    else
-        avgpool2_kernel<T, 1><<<flat_blocks(len), 256, 0, s>>>(x, y, batch, n, c);
-    return cudaGetLastError();
+        return launch_chained(avgpool2_kernel<T, 2>, flat_blocks(len / 2), 256, 0, s, true, x, y, batch, n, c);
+    return launch_chained(avgpool2_kernel<T, 1>, flat_blocks(len), 256, 0, s, true, x, y, batch, n, c);
 }
 
 cudaError_t avgpool2_backward(const float *dy, float *dx, int batch, int n, int c, cudaStream_t s)
@@ -1730,10 +1735,8 @@ cudaError_t up2_add(const T *x, const T *skip, T *y, int batch, int n, int c, cu
     if (c % 4 != 0) return cudaErrorInvalidValue;
     const long long len = static_cast<long long>(batch) * 8LL * n * n * n * (c / 4);
     if (std::is_same_v<T, __nv_bfloat16> && c % 8 == 0)
-        up2_add_kernel<T, 2><<<flat_blocks(len / 2), 256, 0, s>>>(x, skip, y, batch, n, c);
-    else
-        up2_add_kernel<T, 1><<<flat_blocks(len), 256, 0, s>>>(x, skip, y, batch, n, c);
-    return cudaGetLastError();
+        return launch_chained(up2_add_kernel<T, 2>, flat_blocks(len / 2), 256, 0, s, true, x, skip, y, batch, n, c);
+    return launch_chained(up2_add_kernel<T, 1>, flat_blocks(len), 256, 0, s, true, x, skip, y, batch, n, c);
 }
 
 cudaError_t up2_backward(const float *dy, float *dx, int batch, int n, int c, cudaStream_t s)
@@ -1788,9 +1791,7 @@ cudaError_t features(const double *ra, const int *wall, T *out, int batch, int n
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
     // one wave of blocks: each pays the FP64 logarithm once
     const unsigned blocks = std::min(flat_blocks(static_cast<long long>(batch) * n * n * n), 152u * 8u);
-    features_kernel<T><<<blocks, 256, smem, s>>>(
-        ra, wall, out, batch, n);
-    return cudaGetLastError();
+    return launch_chained(features_kernel<T>, blocks, 256, smem, s, true, ra, wall, out, batch, n);
 }
 
 template <typename T>
@@ -1836,7 +1837,7 @@ cudaError_t target_from_fields(const float *u, const float *theta, const float *
 // explicit instantiations for float and bfloat16 storage
 #define DMRT_NN_INST(T)                                                                        \
     template cudaError_t conv3d<T, T, T>(const T *, const T *, const float *, T *, int, int, int, \
-                                         int, int, int, cudaStream_t);                          \
+                                         int, int, int, cudaStream_t, bool);                    \
     template cudaError_t conv3d_wgrad<T>(const T *, const float *, float *, float *, size_t, int, \
                                          int, int, int, int, cudaStream_t);                     \
     template cudaError_t act_backward<T>(const T *, float *, long long, cudaStream_t);          \
@@ -1864,11 +1865,11 @@ DMRT_NN_INST(__nv_bfloat16)
 template cudaError_t conv3d<__nv_bfloat16, __nv_bfloat16, float>(const __nv_bfloat16 *,
                                                                 const __nv_bfloat16 *, const float *,
                                                                 float *, int, int, int, int, int, int,
-                                                                cudaStream_t);
+                                                                cudaStream_t, bool);
 // input gradients of bf16 layers: FP32 gradients through bf16 weights
 template cudaError_t conv3d<float, __nv_bfloat16, float>(const float *, const __nv_bfloat16 *,
                                                         const float *, float *, int, int, int, int,
-                                                        int, int, cudaStream_t);
+                                                        int, int, cudaStream_t, bool);
 
 }  // namespace nn
 }  // namespace lbm

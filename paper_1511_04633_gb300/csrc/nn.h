@@ -8,15 +8,43 @@
 namespace lbm {
 namespace nn {
 
+// The network's kernels follow one another with programmatic dependent
+// launch: the next kernel's blocks start, and set up what does not depend on
+// the one before (barriers, TMEM, weights), while that one drains.  A kernel
+// launched so calls chain_wait() before it touches activations or gradients
+// and chain_release() after it, never before: whatever the next kernel
+// does ahead of its own wait then comes after the kernel before this one, and
+// weights are always older than that.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool chained,
+                                  A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Input features per voxel (see features_kernel).
 constexpr int kFeatures = 8;
 
 // y = act(conv_k(x, w) + bias), k in {1, 3}, n a multiple of 8; act: 0 none,
 // 1 leaky ReLU (slope 0.1).  bias may be null.  bfloat16 x and w (cin a
-// multiple of 8) run on tensor cores; other types on CUDA cores.
+// multiple of 8) run on tensor cores; other types on CUDA cores.  chained:
+// w and bias are older than the kernel launched last on s (launch_chained).
 template <typename TI, typename TW, typename TO>
 cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch, int n, int cin,
-                   int cout, int k, int act, cudaStream_t s);
+                   int cout, int k, int act, cudaStream_t s, bool chained = false);
 
 // The 3^3 convolutions of bfloat16 x and w on the tcgen05 tensor cores
 // (conv_umma.cu): taken where the channel counts are multiples of 16 (cin
@@ -24,7 +52,7 @@ cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch
 bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout);
 template <typename TO>
 cudaError_t conv3d_umma(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
-                        int cin, int cout, int act, cudaStream_t s);
+                        int cin, int cout, int act, cudaStream_t s, bool chained);
 
 // dw (FP32, [tap][cout][cin]) of conv3d; scratch holds the per-chunk partials.
 template <typename TI>

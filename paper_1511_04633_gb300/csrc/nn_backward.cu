@@ -63,6 +63,8 @@ __global__ void __launch_bounds__(kThreads)
                        const __nv_bfloat16 *__restrict__ yout, __nv_bfloat16 *__restrict__ dyn, unsigned len4, int n,
                        int c4, float *__restrict__ partials)
 {
+    chain_wait();
+    chain_release();
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     const int c = 4 * c4;
     for (unsigned i = blockIdx.x * kThreads + threadIdx.x; i < len4; i += gridDim.x * kThreads) {
@@ -127,6 +129,8 @@ __global__ void __launch_bounds__(kThreads)
     __shared__ float ws[kHeadOut][kHeadIn];
     for (int e = threadIdx.x; e < kHeadOut * kHeadIn; e += kThreads) ws[e / kHeadIn][e % kHeadIn] = __bfloat162float(w[e]);
     __syncthreads();
+    chain_wait();
+    chain_release();
     constexpr int C = kHeadIn / 2;  // two threads per voxel, eight channels each
     const int c0 = C * (threadIdx.x & 1);
     const float scale = 2.0f / static_cast<float>(voxels * kHeadOut);
@@ -223,6 +227,8 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads) sum_all_kernel(const __grid_constant__ SumList list)
 {
     __shared__ float red[kThreads];
+    chain_wait();
+    chain_release();
     const int b = static_cast<int>(blockIdx.x);
     if (b == list.first[list.count]) {
         __shared__ double redd[kThreads];
@@ -277,6 +283,8 @@ __global__ void __launch_bounds__(kThreads)
     for (int e = threadIdx.x; e < kHeadOut * kHeadIn; e += kThreads) ws[e / kHeadIn][e % kHeadIn] = __bfloat162float(w[e]);
     if (threadIdx.x < kHeadOut) bs[threadIdx.x] = bias[threadIdx.x];
     __syncthreads();
+    chain_wait();
+    chain_release();
     const long long v = blockIdx.x * static_cast<long long>(kThreads) + threadIdx.x;
     if (v >= voxels) return;
     float x[kHeadIn];
@@ -307,6 +315,8 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     flip_all_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bfloat16 *__restrict__ wt, const __grid_constant__ FlipList list)
 {
+    chain_wait();
+    chain_release();
     const int i = static_cast<int>(blockIdx.x * kThreads + threadIdx.x);
     if (i >= list.first[list.count]) return;
     int k = 0;
@@ -327,15 +337,15 @@ cudaError_t grad_narrow(GradSource src, const float *g, const float *h, const __
     const unsigned l = static_cast<unsigned>(len4);
     switch (src) {
     case GradSource::kPlain:
-        grad_narrow_kernel<GradSource::kPlain><<<kGradBlocks, kThreads, 0, s>>>(g, h, yout, dyn, l, n, c / 4, partials);
-        break;
+        return launch_chained(grad_narrow_kernel<GradSource::kPlain>, kGradBlocks, kThreads, 0, s, true, g, h, yout, dyn, l, n,
+                              c / 4, partials);
     case GradSource::kUp2:
-        grad_narrow_kernel<GradSource::kUp2><<<kGradBlocks, kThreads, 0, s>>>(g, h, yout, dyn, l, n, c / 4, partials);
-        break;
+        return launch_chained(grad_narrow_kernel<GradSource::kUp2>, kGradBlocks, kThreads, 0, s, true, g, h, yout, dyn, l, n,
+                              c / 4, partials);
     default:
-        grad_narrow_kernel<GradSource::kPool><<<kGradBlocks, kThreads, 0, s>>>(g, h, yout, dyn, l, n, c / 4, partials);
+        return launch_chained(grad_narrow_kernel<GradSource::kPool>, kGradBlocks, kThreads, 0, s, true, g, h, yout, dyn, l, n,
+                              c / 4, partials);
     }
-    return cudaGetLastError();
 }
 
 template <typename TO>
@@ -344,8 +354,7 @@ cudaError_t head_forward(const __nv_bfloat16 *h, const __nv_bfloat16 *w, const f
 {
     const long long blocks = (voxels + kThreads - 1) / kThreads;
     if (blocks >= (1LL << 31)) return cudaErrorInvalidValue;
-    head_forward_kernel<TO><<<static_cast<unsigned>(blocks), kThreads, 0, s>>>(h, w, bias, y, voxels);
-    return cudaGetLastError();
+    return launch_chained(head_forward_kernel<TO>, static_cast<unsigned>(blocks), kThreads, 0, s, true, h, w, bias, y, voxels);
 }
 template cudaError_t head_forward<float>(const __nv_bfloat16 *, const __nv_bfloat16 *, const float *, float *, long long,
                                          cudaStream_t);
@@ -358,7 +367,8 @@ cudaError_t head_backward(const __nv_bfloat16 *out, const float *target, const _
                           __nv_bfloat16 *dyn, long long voxels, float *partials, double *loss_partials, float *dw,
                           float *db, float *db_before, SumList &sums, cudaStream_t s)
 {
-    head_backward_kernel<<<kHeadBlocks, kThreads, 0, s>>>(out, target, h, w, dyn, voxels, partials, loss_partials);
+    const cudaError_t e = launch_chained(head_backward_kernel, kHeadBlocks, kThreads, 0, s, true, out, target, h, w, dyn,
+                                         voxels, partials, loss_partials);
     constexpr int kw = kHeadOut * kHeadIn;
     sums.add(partials, kHeadSums, dw, kw, kHeadBlocks);
     sums.add(partials + kw, kHeadSums, db, kHeadOut, kHeadBlocks);
@@ -366,7 +376,7 @@ cudaError_t head_backward(const __nv_bfloat16 *out, const float *target, const _
     sums.loss_partials = loss_partials;
     sums.loss_parts = kHeadBlocks;
     sums.loss_scale = 1.0 / static_cast<double>(voxels * kHeadOut);
-    return cudaGetLastError();
+    return e;
 }
 
 void SumList::add(const float *partials, size_t stride, float *out, int len, int chunks)
@@ -386,15 +396,13 @@ void SumList::add(const float *partials, size_t stride, float *out, int len, int
 
 cudaError_t sum_all(const SumList &list, cudaStream_t s)
 {
-    sum_all_kernel<<<list.first[list.count] + 1, kThreads, 0, s>>>(list);
-    return cudaGetLastError();
+    return launch_chained(sum_all_kernel, list.first[list.count] + 1, kThreads, 0, s, true, list);
 }
 
 cudaError_t flip_all(const __nv_bfloat16 *w, __nv_bfloat16 *wt, const FlipList &list, cudaStream_t s)
 {
     const int len = list.first[list.count];
-    flip_all_kernel<<<(len + kThreads - 1) / kThreads, kThreads, 0, s>>>(w, wt, list);
-    return cudaGetLastError();
+    return launch_chained(flip_all_kernel, (len + kThreads - 1) / kThreads, kThreads, 0, s, true, w, wt, list);
 }
 
 }  // namespace nn

@@ -187,7 +187,7 @@ dmrt_status conv_fwd(dmrt_surrogate_t *s, const Layer &L, const void *in, void *
 {
     SCK(s,
         (lbm::nn::conv3d<T, T, T>(static_cast<const T *>(in), W<T>(s, L), B(s, L), static_cast<T *>(out),
-                                  batch, edge(s, L.level), L.cin, L.cout, L.k, L.act, s->stream)),
+                                  batch, edge(s, L.level), L.cin, L.cout, L.k, L.act, s->stream, true)),
         "conv3d");
     return DMRT_OK;
 }
@@ -375,7 +375,7 @@ dmrt_status backward_fused(dmrt_surrogate_t *s, int batch)
         if (gout)
             SCK(s,
                 (lbm::nn::conv3d<B16, B16, float>(s->gnarrow, static_cast<const B16 *>(s->wt) + L.w_off, nullptr, gout,
-                                                  batch, e, L.cout, L.cin, 3, 0, s->stream)),
+                                                  batch, e, L.cout, L.cin, 3, 0, s->stream, true)),
                 "conv3d (input gradient)");
         return DMRT_OK;
     };
