@@ -34,7 +34,6 @@
 //
 // Each wait is bounded; one that runs out sets *err, and the CTA drains its
 // copies and MMAs before it releases its TMEM and exits.
-#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>

@@ -608,25 +608,6 @@ __device__ __forceinline__ void st2<__nv_bfloat16>(__nv_bfloat16 *p, float a, fl
     *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
 }
 
-// Eight consecutive channels in one or two 16-byte stores (p 16-byte aligned).
-template <typename T>
-__device__ __forceinline__ void st8(T *p, const float *v);
-template <>
-__device__ __forceinline__ void st8<float>(float *p, const float *v)
-{
-    reinterpret_cast<float4 *>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
-    reinterpret_cast<float4 *>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
-}
-template <>
-__device__ __forceinline__ void st8<__nv_bfloat16>(__nv_bfloat16 *p, const float *v)
-{
-    uint4 u;
-    __nv_bfloat162 h[4];
-    for (int i = 0; i < 4; ++i) h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-    memcpy(&u, h, sizeof u);
-    *reinterpret_cast<uint4 *>(p) = u;
-}
-
 // Tensor-core 3^3 convolution (implicit GEMM, mma.m16n8k16, FP32
 // accumulation) over 8 x 8 x 4 voxel tiles: a block owns one tile of one
 // sample and 8 NT output channels.  For every 16 input channels it stages
