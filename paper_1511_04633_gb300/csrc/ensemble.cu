@@ -531,6 +531,8 @@ __global__ void __launch_bounds__(128, kEnsPairBlocks)
 }
 
 // In-place scheme (step_inplace_pair_kernel's two phases) for a shape group.
+// PHASE 2 is phase 1 after a phase 0 that started from the two-buffer layout,
+// which it restores.
 template <typename T, bool SR, int PHASE>
 __global__ void __launch_bounds__(128, kEnsPairBlocks)
     ensemble_group_inplace_pair_kernel(T *__restrict__ buf, const InplaceGeometry SI, const GroupCounters K,
@@ -552,8 +554,11 @@ __global__ void __launch_bounds__(128, kEnsPairBlocks)
     if constexpr (PHASE == 0)
         pull_pair<kRuntimeWall, T>(A + self, TableOffsets{S}, P2, theta_linear(y, S.inv_ny), d, g, M.wall != 1,
                                    M.wall == 2);
-    else
+    else if constexpr (PHASE == 1)
         pull_pair<kRuntimeWall, T>(A + self, LocalOffsets{S.plane}, P2, theta_linear(y, S.inv_ny), d, g,
+                                   M.wall != 1, M.wall == 2);
+    else
+        pull_pair<kRuntimeWall, T>(A + self, LocalOppOffsets{S.plane}, P2, theta_linear(y, S.inv_ny), d, g,
                                    M.wall != 1, M.wall == 2);
     const unsigned r01 = SR ? pair_bits_salted(self, salt) : 0u;
     T *Dp = A + self;
@@ -564,6 +569,8 @@ __global__ void __launch_bounds__(128, kEnsPairBlocks)
         const unsigned r = SR ? plane_bits<q>(r01) : 0u;
         if constexpr (PHASE == 1) {
             store2<T, SR>(Dp + plane_opp<q>() * plane, v, r);
+        } else if constexpr (PHASE == 2) {
+            store2<T, SR>(Dp + q * plane, v, r);
         } else {
             constexpr int ex = plane_ex<q>(), ey = plane_ey<q>(), ez = plane_ez<q>();
             bool lyz = false;  // the link leaves through a y or z face
@@ -876,7 +883,8 @@ cudaError_t launch_ensemble_inplace(int storage, bool stochastic, void *buf, int
 
 // One shape group's chunk: grid (tiles along x, tiles along y, nz * members)
 // of bx x (128 / bx) threads; phase < 0: two-buffer step from src to dst,
-// else the in-place phase on src.
+// else the in-place phase on src (0 and 2, with the tables of
+// fill_ab_inplace_geometry: two steps of a two-buffer state within src).
 cudaError_t launch_ensemble_group(int storage, bool stochastic, const void *src, void *dst, int phase,
                                   const InplaceGeometry &SI, const GroupTable &P, int bx, const GroupCounters &K,
                                   cudaStream_t s, bool pdl)
@@ -905,14 +913,17 @@ cudaError_t launch_ensemble_group(int storage, bool stochastic, const void *src,
             return cudaLaunchKernelEx(&cfg, ensemble_group_pair_kernel<T, false>, a, b, S, K, P);
         }
         T *A = static_cast<T *>(const_cast<void *>(src));
-        auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, A, SI, K, P); };
+        auto by_phase = [&](auto sr) {
+            constexpr bool SR = decltype(sr)::value;
+            auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, A, SI, K, P); };
+            if (phase == 0) return go(ensemble_group_inplace_pair_kernel<T, SR, 0>);
+            if (phase == 1) return go(ensemble_group_inplace_pair_kernel<T, SR, 1>);
+            return go(ensemble_group_inplace_pair_kernel<T, SR, 2>);
+        };
         if constexpr (!std::is_same_v<T, float>) {
-            if (stochastic)
-                return phase == 0 ? go(ensemble_group_inplace_pair_kernel<T, true, 0>)
-                                  : go(ensemble_group_inplace_pair_kernel<T, true, 1>);
+            if (stochastic) return by_phase(std::true_type{});
         }
-        return phase == 0 ? go(ensemble_group_inplace_pair_kernel<T, false, 0>)
-                          : go(ensemble_group_inplace_pair_kernel<T, false, 1>);
+        return by_phase(std::false_type{});
     });
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -993,6 +1004,7 @@ struct dmrt_ensemble {
     std::vector<int> group_bx;
     std::vector<GroupChunk> chunks;
     bool grouped = false;  // steps by shape groups (else by the tables)
+    bool by_twos = false;  // two buffers, plain steps in place by twos (groups)
     // Captured intervals of shape groups run one chain of launches per
     // chunk, concurrently (side streams, fork / join events), each with its
     // own pair of step counters.
@@ -1250,7 +1262,7 @@ void build_groups(dmrt_ensemble_t *e, const std::vector<lbm::BlockTile> &map)
         G.inv_ny = D.inv_ny;
         lbm::InplaceGeometry SI{};
         if (e->inplace) lbm::fill_inplace_geometry(G, SI);
-        else lbm::fill_step_geometry(G, SI.load);
+        else lbm::fill_ab_inplace_geometry(G, SI);
         e->group_geom.push_back(SI);
         e->group_bx.push_back(D.bx);
         const size_t per = static_cast<size_t>(std::min(lbm::kGroupMembers, 65535 / D.nz));
@@ -1271,6 +1283,22 @@ void build_groups(dmrt_ensemble_t *e, const std::vector<lbm::BlockTile> &map)
     }
 }
 
+// Do the plain steps of shape groups pay in place by twos, within one of the
+// two buffers?  Half the memory is touched: FP32 gains where one buffer stays
+// in L2 (129 MB) and two do not, and nothing in HBM; the 16-bit group kernels
+// are also faster in place in HBM, where they store to the lines they loaded.
+// Measured on GB300, per step, between the buffers -> in place, by the bytes
+// of one buffer: FP32 27 MB 6.4 -> 6.6 us, 46 MB 11.9 -> 10.6, 69 MB 21.3 ->
+// 14.9, 92 MB 28.6 -> 25.3, 109 MB 33.7 -> 32.0, 115 MB 35.2 -> 37.1, 2.1 GB
+// 616 -> 630; BF16 35 MB 15.2 -> 15.4, 41 MB 14.4 -> 14.2, 46 MB 21.5 ->
+// 20.0, 54 MB 22.8 -> 18.1, 109 MB 43.7 -> 40.6, 1.1 GB 411 -> 391 (FP16 414
+// -> 400), 1.5 GB 556 -> 526.
+bool steps_by_twos(const dmrt_ensemble_t *e)
+{
+    const long long bytes = e->total_elems * lbm::storage_bytes(e->storage);
+    return bytes >= 45000000ll && (e->storage != DMRT_STORE_F32 || bytes <= 110000000ll);
+}
+
 dmrt_status upload_layout(dmrt_ensemble_t *e, const std::vector<lbm::BlockTile> &map)
 {
     // captured graphs hold the previous launches' tables
@@ -1284,6 +1312,7 @@ dmrt_status upload_layout(dmrt_ensemble_t *e, const std::vector<lbm::BlockTile> 
         build_groups(e, map);
         e->grouped = e->chunks.size() <= kMaxGroupLaunches;
     }
+    e->by_twos = e->grouped && !e->inplace && steps_by_twos(e);
     if (map.size() > e->blockmap_cap) {
         if (e->d_blockmap) cudaFree(e->d_blockmap);
         e->d_blockmap = nullptr;
@@ -1352,6 +1381,24 @@ cudaError_t launch_group_chunk(dmrt_ensemble_t *e, size_t i, int from, cudaStrea
                                       e->group_geom[ch.group], ch.table, e->group_bx[ch.group], K, s, e->use_pdl);
 }
 
+// The first (phase 0) or second (phase 2) of two steps of chunk i of a
+// two-buffer ensemble within buffer `from`: phase 0 leaves every value where
+// phase 2 finds it in the cell's own slots, and phase 2 restores the
+// two-buffer layout.  The step between them has the second word of the
+// buffer's tail (in a chain: of the chain's pair) as its counter; without
+// chains, phase 0 of every chunk comes before phase 2 of any.
+cudaError_t launch_group_chunk_within(dmrt_ensemble_t *e, size_t i, int from, int phase, cudaStream_t s, bool chain)
+{
+    const auto &ch = e->chunks[i];
+    unsigned *tail = step_counter(e, from);
+    unsigned *even = chain ? e->chain_ctr + 2 * i + from : tail;
+    unsigned *odd = chain ? e->chain_ctr + 2 * i + (from ^ 1) : tail + 1;
+    const lbm::GroupCounters K = phase == 0 ? lbm::GroupCounters{even, odd, nullptr}
+                                            : lbm::GroupCounters{odd, even, chain ? tail : nullptr};
+    return lbm::launch_ensemble_group(e->storage, e->stochastic, e->buf[from], nullptr, phase,
+                                      e->group_geom[ch.group], ch.table, e->group_bx[ch.group], K, s, e->use_pdl);
+}
+
 // One step of every member from state `from`; with `res` a residual point of
 // that state is taken first (the points are the states that the last step
 // of every K-step interval starts from, as in a single cavity).
@@ -1380,6 +1427,27 @@ cudaError_t launch_one_step(dmrt_ensemble_t *e, int from, bool res = false)
         if (c != cudaSuccess) return c;
     }
     return cudaSuccess;
+}
+
+// The next step or two of every member from state `ph` (which follows), of
+// which the last one before a residual point may be `until_res` steps away;
+// at most `most`.  *done: the steps launched.
+cudaError_t launch_steps(dmrt_ensemble_t *e, int &ph, long until_res, long most, long *done)
+{
+    if (e->by_twos && most >= 2 && until_res > 2) {
+        *done = 2;
+        for (int phase : {0, 2}) {
+            for (size_t i = 0; i < e->chunks.size(); ++i) {
+                const cudaError_t c = launch_group_chunk_within(e, i, ph, phase, e->stream, false);
+                if (c != cudaSuccess) return c;
+            }
+        }
+        return cudaSuccess;
+    }
+    *done = 1;
+    const cudaError_t c = launch_one_step(e, ph, until_res == 1);
+    ph ^= 1;
+    return c;
 }
 
 // Side streams, events and chain counters for concurrent chains.
@@ -1431,13 +1499,22 @@ bool capture_chains(dmrt_ensemble_t *e, int start)
         e->graph_extra = 1;
     }
     if (!fork()) return false;
-    for (long s = 0; s < e->K; ++s) {
+    for (long s = 0; s < e->K;) {
         if (s == e->K - 1) {
             if (!join() || launch_residual_point(e, cur) != cudaSuccess || !fork()) return false;
         }
-        for (int i = 0; i < n; ++i)
-            if (launch_group_chunk(e, static_cast<size_t>(i), cur, e->side[i], true) != cudaSuccess) return false;
-        cur ^= 1;
+        const bool twice = e->by_twos && s + 2 < e->K;
+        for (int i = 0; i < n; ++i) {
+            const size_t c = static_cast<size_t>(i);
+            if (!twice) {
+                if (launch_group_chunk(e, c, cur, e->side[i], true) != cudaSuccess) return false;
+                continue;
+            }
+            for (int phase : {0, 2})
+                if (launch_group_chunk_within(e, c, cur, phase, e->side[i], true) != cudaSuccess) return false;
+        }
+        if (!twice) cur ^= 1;
+        s += twice ? 2 : 1;
     }
     return join();
 }
@@ -1456,10 +1533,8 @@ bool capture_interval(dmrt_ensemble_t *e, int start)
         ok = capture_chains(e, start);
     } else {
         e->graph_extra = 0;
-        for (long s = 0; s < e->K && ok; ++s) {
-            ok = launch_one_step(e, cur, s == e->K - 1) == cudaSuccess;
-            cur ^= 1;
-        }
+        for (long s = 0, did = 0; s < e->K && ok; s += did)
+            ok = launch_steps(e, cur, e->K - s, e->K - s, &did) == cudaSuccess;
     }
     cudaGraph_t graph = nullptr;
     ok = (cudaStreamEndCapture(e->stream, &graph) == cudaSuccess) && ok && graph;
@@ -1497,11 +1572,10 @@ dmrt_status run_steps(dmrt_ensemble_t *e, long n)
             }
         }
         bool took = graphed;  // a whole interval ends with a residual point
-        for (long s = 0; s < chunk && !graphed; ++s) {
-            const bool res = (e->steps + s + 1) % e->K == 0;
-            ECK(e, launch_one_step(e, ph, res), "ensemble step");
-            took = took || res;
-            ph ^= 1;
+        for (long s = 0, did = 0; s < chunk && !graphed; s += did) {
+            const long until_res = e->K - (e->steps + s) % e->K;
+            ECK(e, launch_steps(e, ph, until_res, chunk - s, &did), "ensemble step");
+            took = took || until_res == 1;
         }
         e->steps += chunk;
         const long per_step = static_cast<long>(e->grouped ? e->chunks.size() : e->tables.size());  // launches

@@ -57,3 +57,27 @@ def test_bitwise_the_one_cell_kernels(dm, grid, wall, storage, K):
         assert np.array_equal(p, q)
     a.close()
     b.close()
+
+
+# shape groups whose plain steps run in place by twos: two chains of mixed
+# shapes (the rule's FP32 and 16-bit ranges), one chain, one shape in two
+# launches; even and odd residual intervals, graph-replayed and launched singly
+@pytest.mark.parametrize("shapes,each,storage,K", [
+    ([(50, 41, 33), (70, 64, 30)], 3, 0, 6), ([(50, 41, 33), (70, 64, 30)], 5, 1, 7), ([(36, 50, 42)], 12, 2, 5),
+    ([(24, 24, 24)], 70, 1, 2), ([(24, 24, 24), (2, 40, 60)], 65, 2, 4),
+])
+def test_ensembles_bitwise_the_one_cell_kernels(dm, shapes, each, storage, K):
+    cav = [{"grid": shapes[k % len(shapes)], "Ra": 10 ** (3 + 2 * k / 130), "wall": 1 + k % 3}
+           for k in range(each * len(shapes))]
+    a = dm.Ensemble(cav, storage=storage, residual_interval=K)
+    b = dm.Ensemble(cav, storage=storage, residual_interval=K, cells_per_thread=1)
+    for n in (1, 2, 3, 2 * K, K + 3):
+        a.step(n)
+        b.step(n)
+        for k in (0, 1, len(cav) // 2, len(cav) - 1):
+            for p, q in zip(a.populations(k), b.populations(k)):
+                assert np.array_equal(p, q), (n, k)
+    assert np.array_equal(np.asarray(a.residual()), np.asarray(b.residual()))
+    assert np.array_equal(np.asarray(a.nusselt(1)), np.asarray(b.nusselt(1)))
+    a.close()
+    b.close()
