@@ -81,7 +81,9 @@ typedef enum {
 /* How the populations stream (the method is the same; only the memory
  * scheme differs).
  *  AB     : two population buffers; each step pulls from one and writes the
- *           other (2 x 26 values per cell held on the device).
+ *           other (2 x 26 values per cell held on the device).  Sizes whose
+ *           working set then fits L2 (and 16-bit ensembles) take plain steps
+ *           two at a time within one buffer; the values are the same.
  *  INPLACE: one buffer updated in place by two alternating kernels (the AA
  *           access pattern): half the population memory, the same HBM
  *           traffic per step, and bitwise the same results as AB in every
@@ -105,7 +107,9 @@ typedef struct dmrt_opts {
                             * else DMRT_ERR_ARG).  Either streaming scheme.
                             * The stored values are bitwise the same either
                             * way.  Auto takes 2 where allowed; for an
-                            * ensemble, where every member's nx is even. */
+                            * ensemble, where every member's nx is even.  A
+                            * walled cavity with odd nx may then pair cells
+                            * of neighbouring slabs (reported as 1). */
     int pair_loads;        /* how the two-cell kernel of two-buffer 16-bit
                             * storage loads: 0 = auto (direct), 1 = direct
                             * loads, 2 = staged: TMA copies of each plane's
