@@ -913,6 +913,11 @@ dmrt_status dmrt_checkpoint_save(dmrt_t *h, void *dst, long long size)
     p += hd.snap_bytes;
     CK(h, cudaMemcpyAsync(p, h->dres, 8 * sizeof(double), cudaMemcpyDeviceToHost, h->stream), "copy residual");
     CK(h, cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    // a two-buffer state has one counter word; steps taken in place by twos
+    // leave the number of the step between them in the second, which depends
+    // on how the steps were divided among the calls
+    if (!h->inplace)
+        memset(static_cast<char *>(dst) + sizeof hd + hd.pop_bytes - 256 + sizeof(unsigned), 0, sizeof(unsigned));
     return DMRT_OK;
 }
 
