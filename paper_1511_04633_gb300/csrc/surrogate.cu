@@ -15,12 +15,16 @@
 // master weights.  The backward pass is written out by hand below.
 #include <cmath>
 #include <cstdarg>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <new>
 #include <string>
 #include <type_traits>
 #include <vector>
+
+#include <cuda.h>
+#include <cudaTypedefs.h>
 
 #include "dmrt.h"
 #include "internal.h"
@@ -482,6 +486,32 @@ dmrt_status check_batch(dmrt_surrogate_t *s, int batch, const double *ra, const 
     return DMRT_OK;
 }
 
+// May a kernel of the surrogate's device write `bytes` bytes at p?  Known only
+// for one allocation of that device's own memory and FP32 alignment.  All
+// else (memory of another GPU, host memory, an odd address, a range that
+// leaves its allocation) is left to cudaMemcpy, which serves or refuses it.
+bool own_device_memory(const dmrt_surrogate_t *s, const void *p, size_t bytes)
+{
+    static const auto range = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 3020, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return reinterpret_cast<PFN_cuMemGetAddressRange_v3020>(fn);
+    }();
+    cudaPointerAttributes a;
+    if (!range || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    const auto at = reinterpret_cast<uintptr_t>(p);
+    if (a.type != cudaMemoryTypeDevice || a.device != s->device || at % alignof(float) != 0) return false;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return range(&base, &size, static_cast<CUdeviceptr>(at)) == CUDA_SUCCESS && at - base <= size && bytes <= size - (at - base);
+}
+
 template <typename F>
 dmrt_status by_storage(dmrt_surrogate_t *s, F &&f)
 {
@@ -650,15 +680,18 @@ dmrt_status dmrt_surrogate_predict(dmrt_surrogate_t *s, int batch, const double 
     if (st != DMRT_OK) return st;
     SGuard g(s->device);
     const long long len = static_cast<long long>(batch) * voxels(s, 0) * kOut;
+    const bool direct = on_device && own_device_memory(s, out, static_cast<size_t>(len) * sizeof(float));
     st = by_storage(s, [&](auto *tp) -> dmrt_status {
         using T = std::remove_pointer_t<decltype(tp)>;
         dmrt_status r = make_features<T>(s, batch, ra, wall);
         if (r != DMRT_OK) return r;
-        return forward<T>(s, batch, on_device ? out : s->g0);
+        return forward<T>(s, batch, direct ? out : s->g0);
     });
     if (st != DMRT_OK) return st;
-    if (!on_device)
-        SCK(s, cudaMemcpyAsync(out, s->g0, len * 4, cudaMemcpyDeviceToHost, s->stream), "copy prediction");
+    if (!direct)
+        SCK(s, cudaMemcpyAsync(out, s->g0, len * 4, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                               s->stream),
+            "copy prediction");
     SCK(s, cudaStreamSynchronize(s->stream), "cudaStreamSynchronize");
     return DMRT_OK;
 }

@@ -221,3 +221,26 @@ def test_channel_blocks_of_the_small_grid_convolution_give_the_same_bits(env):
     ref = S.leaky(S.conv3d(xs, w.double().cpu().numpy().reshape(27, cout, cin), b.double().cpu().numpy(), 3))
     got = y_small.double().cpu().numpy()
     assert np.abs(got - ref).max() <= 2e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("storage", ["F32", "BF16"])
+def test_prediction_into_memory_no_kernel_can_write(env, storage):
+    """Device addresses that are no FP32 address (2 bytes into an allocation)
+    and pinned host memory are served by a copy, as any other memory."""
+    torch, dm = env
+    sur = dm.Surrogate(16, 1, (16, 32), storage=getattr(dm, "STORE_" + storage), max_batch=2)
+    sur.set_params(inputs.random_weights(sur.param_count, seed=5, scale=0.3))
+    ra, wall = np.array([2e3, 3e5]), np.array([1, 3], np.int32)
+    ref = sur.predict(ra, wall)
+    bytes_ = ref.nbytes
+    raw = torch.zeros(bytes_ + 4, dtype=torch.uint8, device="cuda")
+    pinned = torch.zeros(bytes_, dtype=torch.uint8).pin_memory()
+    for out, at, on_device in ((raw, 0, 1), (raw, 2, 1), (pinned, 0, 0)):
+        raw.zero_()
+        torch.cuda.synchronize()
+        st = dm.load().dmrt_surrogate_predict(sur.s, 2, np.ctypeslib.as_ctypes(ra), np.ctypeslib.as_ctypes(wall),
+                                              out.data_ptr() + at, on_device)
+        assert st == dm.OK
+        assert at == 0 or (int(raw[:at].sum()) == 0 and int(raw[at + bytes_:].sum()) == 0)
+        got = out[at:at + bytes_].cpu().numpy().copy().view(np.float32).reshape(ref.shape)
+        assert np.array_equal(got, ref)
