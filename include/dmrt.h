@@ -177,7 +177,10 @@ dmrt_status dmrt_set_stream(dmrt_t *h, void *stream);
  * compares the fields of the state it pulls with the snapshot of the
  * previous point and reduces the sums of dmrt_residual, in the same pass
  * (a small kernel then adds the block sums).  Asynchronous: returns once the
- * work is queued. */
+ * work is queued.  If CUDA refuses a launch between two steps taken in place
+ * (DMRT_STREAM_AB), the state is lost: every call that reads or steps it
+ * returns DMRT_ERR_CUDA until a state is set or loaded (an ensemble: until
+ * every member's fields are). */
 dmrt_status dmrt_step(dmrt_t *h, long n);
 
 /* Wait for the handle's queued work; reports deferred CUDA errors. */

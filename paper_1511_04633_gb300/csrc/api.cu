@@ -44,6 +44,7 @@ struct dmrt {
     lbm::InplaceGeometry SI{};
     bool ab_inplace = false;              // two buffers, plain steps in place by twos
     lbm::InplaceGeometry ab_SI{};         // and their tables
+    bool torn = false;                    // the second of two such steps was not launched: no state to read
     long long device_bytes = 0;           // device memory held by the handle
     float *snap = nullptr;                // residual snapshot: theta, u (4 planes)
     double *partials = nullptr;           // reduction scratch (Nu rows; residual block partials)
@@ -114,6 +115,14 @@ dmrt_status cuda_fail(dmrt_t *h, cudaError_t e, const char *what)
         if (e_ != cudaSuccess) return cuda_fail(h, e_, what); \
     } while (0)
 
+// The state can be read and stepped: not after two steps in place of which
+// only the first was launched, until a new state is set.
+#define WHOLE(h)                                                                                                  \
+    do {                                                                                                          \
+        if ((h)->torn)                                                                                            \
+            return fail(h, DMRT_ERR_CUDA, "an earlier step failed between two launches; set or load a new state"); \
+    } while (0)
+
 // Keeps the handle's device current for the duration of a call.
 struct DeviceGuard {
     int prev = -1;
@@ -182,10 +191,12 @@ cudaError_t launch_one_step(dmrt_t *h, int ph, bool res)
                                        reinterpret_cast<unsigned *>(h->dres + 7), h->K, h->dres, h->stream);
 }
 
-// Two plain steps of a two-buffer state in place, on its own buffer.
-cudaError_t launch_two_steps(dmrt_t *h, int ph)
+// Two plain steps of a two-buffer state in place, on its own buffer.  *torn:
+// the first went out and the second did not.
+cudaError_t launch_two_steps(dmrt_t *h, int ph, bool *torn)
 {
     for (int phase : {0, 2}) {
+        *torn = phase == 2;
         const cudaError_t e =
             h->split ? lbm::launch_step_inplace_split(h->wall, h->storage, h->stochastic, h->buf[ph], phase, h->ab_SI,
                                                       h->G, h->C, h->stream, h->use_pdl)
@@ -193,17 +204,19 @@ cudaError_t launch_two_steps(dmrt_t *h, int ph)
                                                      h->G, h->C, h->stream, h->use_pdl);
         if (e != cudaSuccess) return e;
     }
+    *torn = false;
     return cudaSuccess;
 }
 
 // The next step or two from state `ph` (which follows), of which the last may
 // come `until_res` steps from now, when a residual point is due; at most
-// `most`.  *done: the steps launched.
-cudaError_t launch_steps(dmrt_t *h, int &ph, long until_res, long most, long *done)
+// `most`.  *done: the steps launched; *torn as in launch_two_steps.
+cudaError_t launch_steps(dmrt_t *h, int &ph, long until_res, long most, long *done, bool *torn)
 {
+    *torn = false;
     if (h->ab_inplace && most >= 2 && until_res > 2) {
         *done = 2;
-        return launch_two_steps(h, ph);
+        return launch_two_steps(h, ph, torn);
     }
     *done = 1;
     const cudaError_t e = launch_one_step(h, ph, until_res == 1);
@@ -291,8 +304,9 @@ bool capture_interval(dmrt_t *h, int start)
         return false;
     }
     int ph = start;
-    bool ok = true;
-    for (long s = 0, m = 0; s < h->K && ok; s += m) ok = launch_steps(h, ph, h->K - s, h->K - s, &m) == cudaSuccess;
+    bool ok = true, torn;  // (nothing runs during the capture)
+    for (long s = 0, m = 0; s < h->K && ok; s += m)
+        ok = launch_steps(h, ph, h->K - s, h->K - s, &m, &torn) == cudaSuccess;
     cudaGraph_t graph = nullptr;
     ok = (cudaStreamEndCapture(h->stream, &graph) == cudaSuccess) && ok && graph;
     cudaGraphExec_t exec = nullptr;
@@ -311,6 +325,7 @@ bool capture_interval(dmrt_t *h, int start)
 // a residual point.  A whole interval of K steps replays a captured graph.
 dmrt_status run_steps(dmrt_t *h, long n)
 {
+    if (n > 0) WHOLE(h);
     long done = 0;
     while (done < n) {
         long until_res = h->K - (h->steps % h->K);
@@ -339,7 +354,7 @@ dmrt_status run_steps(dmrt_t *h, long n)
         }
         for (long s = 0, m = 0; s < chunk && !graphed; s += m) {
             const long to_go = h->K - h->steps % h->K;
-            CK(h, launch_steps(h, ph, to_go, chunk - s, &m), "step kernel");
+            CK(h, launch_steps(h, ph, to_go, chunk - s, &m, &h->torn), "step kernel");
             h->steps += m;
             h->step_launches += m;
             h->total_launches += m;
@@ -617,6 +632,7 @@ dmrt_status dmrt_sync(dmrt_t *h)
 dmrt_status dmrt_fields(dmrt_t *h, float *rho, float *u, float *theta, int on_device)
 {
     if (!h) return DMRT_ERR_ARG;
+    WHOLE(h);
     DeviceGuard dg(h->device);
     const size_t cells = static_cast<size_t>(cell_count(h->G));
     float *drho = rho, *du = u, *dth = theta;
@@ -650,6 +666,7 @@ dmrt_status dmrt_nusselt(dmrt_t *h, int wall, double out[3])
     if (!h || !out) return DMRT_ERR_ARG;
     if (wall != 0 && wall != 1) return fail(h, DMRT_ERR_ARG, "dmrt_nusselt: wall must be 0 or 1");
     if (h->G.ny < 2) return fail(h, DMRT_ERR_ARG, "dmrt_nusselt: needs ny >= 2");
+    WHOLE(h);
     DeviceGuard dg(h->device);
     CK(h,
        lbm::launch_nusselt(h->wall, h->storage, h->buf[h->cur], state_geometry(h), wall, nullptr, h->partials,
@@ -667,6 +684,7 @@ dmrt_status dmrt_nusselt_flux(dmrt_t *h, int wall, double out[3])
     if (!h || !out) return DMRT_ERR_ARG;
     if (wall != 0 && wall != 1) return fail(h, DMRT_ERR_ARG, "dmrt_nusselt_flux: wall must be 0 or 1");
     if (h->wall == DMRT_WALL_PERIODIC) return fail(h, DMRT_ERR_ARG, "dmrt_nusselt_flux: needs walls");
+    WHOLE(h);
     DeviceGuard dg(h->device);
     CK(h,
        lbm::launch_nusselt_flux(h->storage, h->buf[h->cur], state_geometry(h), wall, h->alpha, nullptr, h->partials, h->dnu,
@@ -683,6 +701,7 @@ dmrt_status dmrt_nusselt_local(dmrt_t *h, int wall, float *local, int on_device)
     if (!h || !local) return DMRT_ERR_ARG;
     if (wall != 0 && wall != 1) return fail(h, DMRT_ERR_ARG, "dmrt_nusselt_local: wall must be 0 or 1");
     if (h->G.ny < 2) return fail(h, DMRT_ERR_ARG, "dmrt_nusselt_local: needs ny >= 2");
+    WHOLE(h);
     DeviceGuard dg(h->device);
     const size_t n = static_cast<size_t>(h->G.nx) * h->G.nz;
     float *dst = local;
@@ -777,6 +796,7 @@ dmrt_status dmrt_set_populations(dmrt_t *h, const float *f, const float *g, int 
     CK(h, lbm::launch_set_populations(h->storage, df, dg_, h->buf[h->cur], state_geometry(h), periodic(h),
                                       h->stream),
        "set kernel");
+    h->torn = false;
     h->total_launches++;
     {
         dmrt_status st = reset_residual(h);
@@ -790,6 +810,7 @@ dmrt_status dmrt_get_populations(dmrt_t *h, float *f, float *g, int on_device)
 {
     if (!h) return DMRT_ERR_ARG;
     if (!f && !g) return DMRT_OK;
+    WHOLE(h);
     DeviceGuard dg(h->device);
     const size_t cells = static_cast<size_t>(cell_count(h->G));
     float *df = f, *dg_ = g;
@@ -844,6 +865,7 @@ dmrt_status dmrt_init_fields(dmrt_t *h, const float *rho, const float *u, const 
     CK(h, lbm::launch_init_fields(h->storage, dr, du, dt, h->buf[h->cur], state_geometry(h), periodic(h),
                                   h->stream),
        "init kernel");
+    h->torn = false;
     h->total_launches++;
     {
         dmrt_status st = reset_residual(h);
@@ -884,6 +906,7 @@ long long dmrt_checkpoint_size(const dmrt_t *h)
 dmrt_status dmrt_checkpoint_save(dmrt_t *h, void *dst, long long size)
 {
     if (!h || !dst || size < dmrt_checkpoint_size(h)) return DMRT_ERR_ARG;
+    WHOLE(h);
     DeviceGuard dg(h->device);
     CheckpointHeader hd{};
     memcpy(hd.magic, kMagic, 8);
@@ -943,6 +966,7 @@ dmrt_status dmrt_checkpoint_load(dmrt_t *h, const void *src, long long size)
     p += hd.snap_bytes;
     CK(h, cudaMemcpyAsync(h->dres, p, 8 * sizeof(double), cudaMemcpyHostToDevice, h->stream), "copy residual");
     CK(h, cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    h->torn = false;
     h->steps = hd.steps;
     h->snaps = hd.snaps;
     h->parity = hd.parity;

@@ -1005,6 +1005,9 @@ struct dmrt_ensemble {
     std::vector<GroupChunk> chunks;
     bool grouped = false;  // steps by shape groups (else by the tables)
     bool by_twos = false;  // two buffers, plain steps in place by twos (groups)
+    // members whose state was lost because a launch within such a pair of
+    // steps failed, until a new one is set (empty: none)
+    std::vector<char> torn;
     // Captured intervals of shape groups run one chain of launches per
     // chunk, concurrently (side streams, fork / join events), each with its
     // own pair of step counters.
@@ -1072,6 +1075,11 @@ dmrt_status ecuda(dmrt_ensemble_t *e, cudaError_t c, const char *what)
 {
     return efail(e, c == cudaErrorMemoryAllocation ? DMRT_ERR_OOM : DMRT_ERR_CUDA, "%s: %s (%s)",
                  what, cudaGetErrorName(c), cudaGetErrorString(c));
+}
+
+dmrt_status state_lost(dmrt_ensemble_t *e)
+{
+    return efail(e, DMRT_ERR_CUDA, "an earlier step failed between its launches; set new fields for every member");
 }
 
 #define ECK(e, call, what)                                   \
@@ -1431,17 +1439,21 @@ cudaError_t launch_one_step(dmrt_ensemble_t *e, int from, bool res = false)
 
 // The next step or two of every member from state `ph` (which follows), of
 // which the last one before a residual point may be `until_res` steps away;
-// at most `most`.  *done: the steps launched.
-cudaError_t launch_steps(dmrt_ensemble_t *e, int &ph, long until_res, long most, long *done)
+// at most `most`.  *done: the steps launched; *torn: a launch within two
+// steps in place failed after others of them had gone out.
+cudaError_t launch_steps(dmrt_ensemble_t *e, int &ph, long until_res, long most, long *done, bool *torn)
 {
+    *torn = false;
     if (e->by_twos && most >= 2 && until_res > 2) {
         *done = 2;
         for (int phase : {0, 2}) {
             for (size_t i = 0; i < e->chunks.size(); ++i) {
                 const cudaError_t c = launch_group_chunk_within(e, i, ph, phase, e->stream, false);
                 if (c != cudaSuccess) return c;
+                *torn = true;
             }
         }
+        *torn = false;
         return cudaSuccess;
     }
     *done = 1;
@@ -1533,8 +1545,9 @@ bool capture_interval(dmrt_ensemble_t *e, int start)
         ok = capture_chains(e, start);
     } else {
         e->graph_extra = 0;
+        bool torn;  // (nothing runs during the capture)
         for (long s = 0, did = 0; s < e->K && ok; s += did)
-            ok = launch_steps(e, cur, e->K - s, e->K - s, &did) == cudaSuccess;
+            ok = launch_steps(e, cur, e->K - s, e->K - s, &did, &torn) == cudaSuccess;
     }
     cudaGraph_t graph = nullptr;
     ok = (cudaStreamEndCapture(e->stream, &graph) == cudaSuccess) && ok && graph;
@@ -1552,6 +1565,7 @@ bool capture_interval(dmrt_ensemble_t *e, int start)
 
 dmrt_status run_steps(dmrt_ensemble_t *e, long n)
 {
+    if (n > 0 && !e->torn.empty()) return state_lost(e);
     long done = 0;
     while (done < n) {
         const long chunk = std::min(n - done, e->K - (e->steps % e->K));
@@ -1574,7 +1588,10 @@ dmrt_status run_steps(dmrt_ensemble_t *e, long n)
         bool took = graphed;  // a whole interval ends with a residual point
         for (long s = 0, did = 0; s < chunk && !graphed; s += did) {
             const long until_res = e->K - (e->steps + s) % e->K;
-            ECK(e, launch_steps(e, ph, until_res, chunk - s, &did), "ensemble step");
+            bool torn;
+            const cudaError_t c = launch_steps(e, ph, until_res, chunk - s, &did, &torn);
+            if (torn) e->torn.assign(static_cast<size_t>(e->count), 1);
+            ECK(e, c, "ensemble step");
             took = took || until_res == 1;
         }
         e->steps += chunk;
@@ -1842,6 +1859,7 @@ dmrt_status dmrt_ensemble_get_stats(dmrt_ensemble_t *e, dmrt_stats *out, int res
 dmrt_status dmrt_ensemble_autotune(dmrt_ensemble_t *e, int trials, char *report, int report_len)
 {
     if (!e || trials < 1) return DMRT_ERR_ARG;
+    if (!e->torn.empty()) return state_lost(e);
     EDeviceGuard dg(e->device);
     ECK(e, cudaStreamSynchronize(e->stream), "cudaStreamSynchronize");
     drop_graphs(e);
@@ -2027,6 +2045,7 @@ dmrt_status dmrt_ensemble_run_to_steady(dmrt_ensemble_t *e, double tol, long max
 dmrt_status dmrt_ensemble_nusselt(dmrt_ensemble_t *e, int wall, double *out)
 {
     if (!e || !out || (wall != 0 && wall != 1)) return DMRT_ERR_ARG;
+    if (!e->torn.empty()) return state_lost(e);
     EDeviceGuard dg(e->device);
     ECK(e,
         lbm::launch_ensemble_nusselt(e->storage, e->buf[e->cur], state_layout(e), e->d_desc, e->count, e->max_nz,
@@ -2044,6 +2063,7 @@ dmrt_status dmrt_ensemble_fields(dmrt_ensemble_t *e, int member, float *rho, flo
                                  float *theta, int on_device)
 {
     if (!e || member < 0 || member >= e->count) return DMRT_ERR_ARG;
+    if (!e->torn.empty() && e->torn[member]) return state_lost(e);
     EDeviceGuard dg(e->device);
     const lbm::CavityDesc &D = e->desc[member];
     const lbm::Geometry G = member_geometry(e, D);
@@ -2092,6 +2112,10 @@ dmrt_status dmrt_ensemble_init_fields(dmrt_ensemble_t *e, int member, const floa
     }
     ECK(e, lbm::launch_init_fields(e->storage, dr, du, dt, member_ptr(e, member, e->cur), G, false, e->stream),
         "init kernel");
+    if (!e->torn.empty()) {
+        e->torn[static_cast<size_t>(member)] = 0;
+        if (std::count(e->torn.begin(), e->torn.end(), 1) == 0) e->torn.clear();
+    }
     e->total_launches++;
     e->snaps = 0;
     ECK(e, cudaMemsetAsync(e->dres + 5 * e->count, 0, sizeof(double), e->stream), "reset residual points");
@@ -2104,6 +2128,7 @@ dmrt_status dmrt_ensemble_get_populations(dmrt_ensemble_t *e, int member, float 
 {
     if (!e || member < 0 || member >= e->count) return DMRT_ERR_ARG;
     if (!f && !g) return DMRT_OK;
+    if (!e->torn.empty() && e->torn[member]) return state_lost(e);
     EDeviceGuard dg(e->device);
     const lbm::CavityDesc &D = e->desc[member];
     const lbm::Geometry G = member_geometry(e, D);

@@ -1,0 +1,94 @@
+"""A launch that the runtime refuses between the two in-place steps of a
+two-buffer state: the handle then has no state, says so, and takes a new one."""
+
+import pytest
+
+from launch_shim import run_child
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+
+
+HELPERS = """
+    def status(f, *a):
+        try:
+            f(*a)
+        except dm.DmrtError as e:
+            return e.status
+        return dm.OK
+
+    start = inputs.random_fields
+"""
+
+
+@pytest.mark.parametrize("grid", [(130, 96, 48), (101, 75, 61)])
+def test_cavity(tmp_path, grid):
+    run_child(tmp_path, HELPERS + f"""
+    grid = {grid}
+    fresh = lambda: dm.Cavity(grid, 1e5, wall_type=2, residual_interval=20)
+    a, ref = fresh(), fresh()
+    for cav in (a, ref):
+        cav.init_fields(*start(grid, 3))
+        cav.step(4)
+    # the first launch refused: nothing has happened
+    shim.shim_refuse(1)
+    assert status(a.step, 4) == dm.ERR_CUDA
+    for p, q in zip(a.fields(), ref.fields()):
+        assert np.array_equal(p, q)
+    # the second one refused: no state
+    shim.shim_refuse(2)
+    assert status(a.step, 4) == dm.ERR_CUDA
+    for f in (a.fields, a.populations, a.save, lambda: a.nusselt(0), lambda: a.nusselt_flux(0), lambda: a.step(1)):
+        assert status(f) == dm.ERR_CUDA
+    # a new state, and a loaded one
+    blob = ref.save()
+    for renew in (lambda cav: cav.init_fields(*start(grid, 5)), lambda cav: cav.load(blob),
+                  lambda cav: cav.set_populations(*[np.copy(v) for v in pops])):
+        pops = ref.populations()
+        shim.shim_refuse(2)
+        status(a.step, 4)
+        assert status(a.fields) == dm.ERR_CUDA
+        shim.shim_refuse(0)
+        renew(a)
+        renew(ref)
+        for cav in (a, ref):
+            cav.step(5)
+        for p, q in zip(a.populations(), ref.populations()):
+            assert np.array_equal(p, q)
+    """)
+
+
+@pytest.mark.parametrize("refused", [2, 3, 4])
+def test_ensemble(tmp_path, refused):
+    run_child(tmp_path, HELPERS + f"""
+    shapes = [(50, 41, 33), (70, 64, 30)]
+    cav = [dict(grid=shapes[k % 2], Ra=1e4 * (1 + k), wall=1 + k % 3) for k in range(6)]
+    a, ref = [dm.Ensemble(cav, residual_interval=20) for _ in range(2)]
+    for e in (a, ref):
+        for k in range(6):
+            e.init_fields(k, *start(cav[k]["grid"], k))
+        e.step(4)
+    shim.shim_refuse(1)
+    assert status(a.step, 4) == dm.ERR_CUDA
+    for k in range(6):
+        assert np.array_equal(a.populations(k)[0], ref.populations(k)[0])
+    shim.shim_refuse({refused})
+    assert status(a.step, 4) == dm.ERR_CUDA
+    for f in (lambda: a.fields(1), lambda: a.populations(5), lambda: a.nusselt(0), lambda: a.step(1), lambda: a.autotune(1)):
+        assert status(f) == dm.ERR_CUDA
+    for k in range(6):
+        assert status(a.step, 1) == dm.ERR_CUDA
+        for e in (a, ref):
+            e.init_fields(k, *start(cav[k]["grid"], 20 + k))
+        assert np.array_equal(a.populations(k)[0], ref.populations(k)[0])
+    for e in (a, ref):
+        e.step(7)
+    for k in range(6):
+        assert np.array_equal(a.populations(k)[0], ref.populations(k)[0])
+    """)
