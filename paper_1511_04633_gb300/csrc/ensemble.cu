@@ -1437,24 +1437,31 @@ cudaError_t launch_one_step(dmrt_ensemble_t *e, int from, bool res = false)
     return cudaSuccess;
 }
 
+// Two plain steps of every member (by_twos) within buffer `b`.  *torn: a
+// launch failed after others of the two steps had gone out.
+cudaError_t launch_two_steps(dmrt_ensemble_t *e, int b, bool *torn)
+{
+    *torn = false;
+    for (int phase : {0, 2}) {
+        for (size_t i = 0; i < e->chunks.size(); ++i) {
+            const cudaError_t c = launch_group_chunk_within(e, i, b, phase, e->stream, false);
+            if (c != cudaSuccess) return c;
+            *torn = true;
+        }
+    }
+    *torn = false;
+    return cudaSuccess;
+}
+
 // The next step or two of every member from state `ph` (which follows), of
 // which the last one before a residual point may be `until_res` steps away;
-// at most `most`.  *done: the steps launched; *torn: a launch within two
-// steps in place failed after others of them had gone out.
+// at most `most`.  *done: the steps launched; *torn as in launch_two_steps.
 cudaError_t launch_steps(dmrt_ensemble_t *e, int &ph, long until_res, long most, long *done, bool *torn)
 {
     *torn = false;
     if (e->by_twos && most >= 2 && until_res > 2) {
         *done = 2;
-        for (int phase : {0, 2}) {
-            for (size_t i = 0; i < e->chunks.size(); ++i) {
-                const cudaError_t c = launch_group_chunk_within(e, i, ph, phase, e->stream, false);
-                if (c != cudaSuccess) return c;
-                *torn = true;
-            }
-        }
-        *torn = false;
-        return cudaSuccess;
+        return launch_two_steps(e, ph, torn);
     }
     *done = 1;
     const cudaError_t c = launch_one_step(e, ph, until_res == 1);
@@ -1865,7 +1872,9 @@ dmrt_status dmrt_ensemble_autotune(dmrt_ensemble_t *e, int trials, char *report,
     drop_graphs(e);
     // In-place ensembles are timed on a scratch copy of their buffer (each
     // launch rewrites its input); two-buffer ones on the live buffers, where
-    // every launch recomputes the same next state from buf[cur].
+    // every launch recomputes the same next state from buf[cur], or, if they
+    // step in place by twos, such pairs within a copy of the state in the
+    // other buffer.
     void *live = e->buf[0];
     void *scratch = nullptr;
     if (e->inplace) {
@@ -1898,22 +1907,32 @@ dmrt_status dmrt_ensemble_autotune(dmrt_ensemble_t *e, int trials, char *report,
     ECK(e, cudaEventCreate(&t0), "cudaEventCreate");
     ECK(e, cudaEventCreate(&t1), "cudaEventCreate");
     int ph = phase(e);
+    const int other = ph ^ 1;
+    if (e->by_twos) {
+        const size_t bytes = static_cast<size_t>(e->total_elems) * lbm::storage_bytes(e->storage) + 256;
+        ECK(e, cudaMemcpyAsync(e->buf[other], e->buf[ph], bytes, cudaMemcpyDeviceToDevice, e->stream),
+            "copy to the other buffer");
+    }
+    // the launches of one timing: a step, or two of them by twos
     auto one = [&]() {
+        bool torn;
+        if (e->by_twos) return launch_two_steps(e, other, &torn);
         const cudaError_t c = launch_one_step(e, ph);
         if (e->inplace) ph ^= 1;  // the scratch state advances
         return c;
     };
-    // time `trials` launches of the current layout of `which`
+    // time `trials` steps (by twos: rounded up) of the current layout of `which`
     auto time_layout = [&](const std::vector<int> &which, float *ms) -> dmrt_status {
         dmrt_status st = upload_layout(e, layout_step(e, which));
         if (st != DMRT_OK) return st;
+        const int per = e->by_twos ? 2 : 1, times = trials / per + trials % per;
         ECK(e, one(), "autotune warm-up");
         ECK(e, cudaEventRecord(t0, e->stream), "cudaEventRecord");
-        for (int t = 0; t < trials; ++t) ECK(e, one(), "autotune launch");
+        for (int t = 0; t < times; ++t) ECK(e, one(), "autotune launch");
         ECK(e, cudaEventRecord(t1, e->stream), "cudaEventRecord");
         ECK(e, cudaEventSynchronize(t1), "cudaEventSynchronize");
         ECK(e, cudaEventElapsedTime(ms, t0, t1), "cudaEventElapsedTime");
-        *ms /= trials;
+        *ms /= static_cast<float>(times * per);
         return DMRT_OK;
     };
     std::map<int, std::vector<int>> groups;  // nx -> members

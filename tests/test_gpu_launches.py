@@ -1,5 +1,6 @@
-"""A launch that the runtime refuses between the two in-place steps of a
-two-buffer state: the handle then has no state, says so, and takes a new one."""
+"""Seen through a stand-in for the launch call: a launch that the runtime refuses
+between the two in-place steps of a two-buffer state (the handle then has no
+state, says so, and takes a new one), and the kernels that the autotuner times."""
 
 import pytest
 
@@ -90,5 +91,35 @@ def test_ensemble(tmp_path, refused):
     for e in (a, ref):
         e.step(7)
     for k in range(6):
+        assert np.array_equal(a.populations(k)[0], ref.populations(k)[0])
+    """)
+
+
+@pytest.mark.parametrize("each,storage,twos", [(3, 0, True), (5, 1, True), (5, 2, True), (1, 0, False)])
+def test_autotune_times_the_kernels_that_step(tmp_path, each, storage, twos):
+    """The step kernels that dmrt_ensemble_autotune launches are those of the
+    interval's plain steps, and the state stays as it was."""
+    run_child(tmp_path, f"""
+    shapes = [(50, 41, 33), (70, 64, 30)]
+    cav = [dict(grid=shapes[k % 2], Ra=1e4 * (1 + k), wall=1 + k % 3) for k in range(2 * {each})]
+    a, ref = [dm.Ensemble(cav, storage={storage}, residual_interval=20) for _ in range(2)]
+    names = lambda: set(n for n in shim.shim_names().decode().split() if "pair_kernel" in n)
+    for e in (a, ref):
+        e.step(5)
+    shim.shim_forget()
+    a.step(4)
+    stepped = names()
+    assert len(stepped) == ({2 if twos else 1}), stepped
+    a.sync()
+    shim.shim_forget()
+    report = a.autotune(3)
+    assert names() == stepped, (names(), stepped)
+    assert "chosen threads=128" in report
+    ref.step(4)
+    for k in range(len(cav)):
+        assert np.array_equal(a.populations(k)[0], ref.populations(k)[0])
+    a.step(18)
+    ref.step(18)
+    for k in range(len(cav)):
         assert np.array_equal(a.populations(k)[0], ref.populations(k)[0])
     """)
