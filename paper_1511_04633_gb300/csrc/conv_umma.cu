@@ -365,10 +365,11 @@ __global__ void __launch_bounds__(kThreads)
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem);  // [kMaxStages]
     uint64_t *empty = full + kMaxStages;                   // [kMaxStages]
-    uint64_t *done = empty + kMaxStages;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1);
+    uint64_t *done = empty + kMaxStages;                   // all chunks are multiplied
+    uint64_t *drained = done + 1;                          // after a failed wait: the MMAs in flight have ended
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(drained + 1);
     float *bs = reinterpret_cast<float *>(smem + 128);
-    static_assert(8 * (2 * kMaxStages + 1) + 4 <= 128 && 128 + 4 * CO <= kHead, "head layout");
+    static_assert(8 * (2 * kMaxStages + 2) + 4 <= 128 && 128 + 4 * CO <= kHead, "head layout");
     constexpr int kVoxels = halo_voxels<PAIR>(R);
     int *offsets = reinterpret_cast<int *>(smem + kHead);  // [voxels]: element offset in the sample, -1 outside
     unsigned char *buf = smem + kHead + table_bytes<PAIR>(R);
@@ -393,6 +394,7 @@ __global__ void __launch_bounds__(kThreads)
             umma::mbar_init(&empty[k], 1);
         }
         umma::mbar_init(done, 1);
+        umma::mbar_init(drained, 1);
     }
     if (warp == 0) umma::tmem_alloc(tslot, kCols);
     if (t < CO) bs[t] = bias ? bias[co0 + t] : 0.f;
@@ -488,10 +490,11 @@ __global__ void __launch_bounds__(kThreads)
         }
         if (!ok) {
             if (leader) atomicExch(err, 1);
-            // MMAs still in flight end before TMEM is released
+            // MMAs still in flight end before TMEM is released (`done` stays
+            // open: the epilogue's wait runs out too and nothing is stored)
             if (issued) {
-                umma::commit(done, leader);
-                (void)umma::mbar_wait(done, 0, kWaitPolls);
+                umma::commit(drained, leader);
+                (void)umma::mbar_wait(drained, 0, kWaitPolls);
             }
         }
     } else {
@@ -524,7 +527,7 @@ __global__ void __launch_bounds__(kThreads)
 
 // ---------------------------------------------------------------- launch
 
-// Device word counting tcgen05 waits that ran out.
+// Device word: not zero once a tcgen05 convolution's wait has run out.
 __device__ int g_umma_err;
 
 int *umma_error_word()

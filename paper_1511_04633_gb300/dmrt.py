@@ -306,7 +306,7 @@ def dmrt_round_to_storage(x, storage: int, rounding: int = ROUND_AUTO, seed: int
 
 
 def dmrt_nn_tensor_core_errors(reset: bool = False) -> int:
-    """Launches of the tcgen05 convolution whose bounded wait ran out."""
+    """Not zero if a bounded wait of a tcgen05 convolution has run out."""
     return int(load().dmrt_nn_tensor_core_errors(1 if reset else 0))
 
 
