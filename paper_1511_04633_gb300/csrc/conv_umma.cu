@@ -37,7 +37,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cstdlib>
 #include <cstring>
 #include <type_traits>
@@ -75,6 +74,42 @@ __device__ __forceinline__ void store8(__nv_bfloat16 *p, const float *v)
     for (int i = 0; i < 4; ++i) h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
     memcpy(&u, h, sizeof u);
     *reinterpret_cast<uint4 *>(p) = u;
+}
+
+// Sixteen consecutive channels (p 16-byte aligned; wide: 32-byte aligned).  A
+// warp's lanes store to 32 different lines, and each store instruction visits
+// every line: 32-byte stores make half the visits of 16-byte ones (48^3 x 6,
+// 16 -> 32 channels, FP32 output: 47.4 -> 42.9 us).
+__device__ __forceinline__ void store32(void *p, const uint4 &a, const uint4 &b)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+                 "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+template <typename TO>
+__device__ __forceinline__ void store16(TO *p, const float *v, bool wide)
+{
+    if (!wide) {
+        store8(p, v);
+        store8(p + 8, v + 8);
+    } else if constexpr (sizeof(TO) == 4) {
+        uint4 u[4];
+        memcpy(u, v, sizeof u);
+        store32(p, u[0], u[1]);
+        store32(p + 8, u[2], u[3]);
+    } else {
+        __nv_bfloat162 h[8];
+        uint4 u[2];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        memcpy(u, h, sizeof u);
+        store32(p, u[0], u[1]);
+    }
+}
+template <typename TO>
+__device__ __forceinline__ bool wide_stores(const TO *y)
+{
+    return (reinterpret_cast<unsigned long long>(y) & 31ull) == 0;
 }
 
 // Copy 16 bytes to shared memory, or zeros if !valid (src stays readable).
@@ -116,7 +151,7 @@ __device__ __forceinline__ void finish16(float (&v)[16], const float *bias, int 
 // MMAs run tap by tap, the K = 16 slices inside.
 constexpr int kRing = 6;
 constexpr int kAcc = 4;
-constexpr int kMinRun = 4;
+constexpr int kMinRun = 2;
 template <int KG>
 constexpr unsigned plane_bytes() { return KG * kHaloRow * 16u; }
 constexpr unsigned kHead = 512;  // mbarriers, TMEM slot, biases
@@ -172,12 +207,23 @@ __global__ void __launch_bounds__(kThreads, KG == 2 ? 4 : 2)
     }
     if (warp == 0) umma::tmem_alloc(tslot, kCols);
     if (t < CO) bs[t] = bias ? bias[t] : 0.f;
-    for (int e = t; e < 27 * KG * CO; e += kThreads) {  // [tap][kg][co] x 16 B
-        const int co = e % CO, kg = (e / CO) % KG, tap = e / (KG * CO);
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (8 * kg < cin)
-            v = *reinterpret_cast<const uint4 *>(w + (static_cast<long long>(tap) * CO + co) * cin + 8 * kg);
-        *reinterpret_cast<uint4 *>(wsm + e * 16) = v;
+    // weights as [tap][kg][co] x 16 B, read in memory order, four loads in flight
+    constexpr int kWeights = 27 * KG * CO;
+#pragma unroll
+    for (int e0 = 0; e0 < kWeights; e0 += 4 * kThreads) {
+        uint4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = e0 + i * kThreads + t, kg = e % KG;
+            v[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (e < kWeights && 8 * kg < cin)
+                v[i] = *reinterpret_cast<const uint4 *>(w + static_cast<long long>(e / KG) * cin + 8 * kg);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = e0 + i * kThreads + t, kg = e % KG, co = e / KG % CO, tap = e / (KG * CO);
+            if (e < kWeights) *reinterpret_cast<uint4 *>(wsm + ((tap * KG + kg) * CO + co) * 16) = v[i];
+        }
     }
     umma::fence_proxy_async_smem();
     umma::fence_before_sync();
@@ -312,8 +358,7 @@ __global__ void __launch_bounds__(kThreads, KG == 2 ? 4 : 2)
                         if (lane == 0) arrive(&acc_empty[buf]);
                     }
                     finish16(v, bs + c16, act);
-                    store8(yo + c16, v);
-                    store8(yo + c16 + 8, v + 8);
+                    store16(yo + c16, v, wide_stores(y));
                 }
             }
             g += run.z_end - run.z_begin;
@@ -512,8 +557,7 @@ __global__ void __launch_bounds__(kThreads)
                     float v[16];
                     umma::ld_32x32b_x16(tmem + (static_cast<uint32_t>(32 * warp) << 16) + i * CO + c16, v);
                     finish16(v, bs + c16, act);
-                    store8(yo + c16, v);
-                    store8(yo + c16 + 8, v + 8);
+                    store16(yo + c16, v, wide_stores(y));
                 }
             }
         } else if (lane == 0) {
@@ -537,25 +581,6 @@ int *umma_error_word()
     return static_cast<int *>(p);
 }
 
-// Streaming multiprocessors of the current device (152 on GB300), asked once
-// per device.
-int sm_count()
-{
-    static std::atomic<int> cached[64];
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) {
-        cudaGetLastError();
-        return 152;
-    }
-    if (dev >= 0 && dev < 64 && (sms = cached[dev].load(std::memory_order_relaxed)) > 0) return sms;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
-        cudaGetLastError();
-        return 152;
-    }
-    if (dev >= 0 && dev < 64) cached[dev].store(sms, std::memory_order_relaxed);
-    return sms;
-}
-
 constexpr unsigned kSmemPerCta = 227u * 1024u, kSmemPerSm = 228u * 1024u;
 
 template <int CO, int KG, typename TO>
@@ -569,26 +594,31 @@ cudaError_t launch_narrow(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const 
     // resident CTAs per SM: shared memory (and 1 KB the runtime reserves per
     // CTA), TMEM columns, the launch bounds
     const int per_sm = std::min({KG == 2 ? 4 : 2, static_cast<int>(kSmemPerSm / (smem + 1024u)), 512 / (kAcc * CO)});
-    // every resident CTA takes an equal share, of at least kMinRun planes
-    // (a run loads two planes more than it computes)
+    // every resident CTA takes an equal share, of at least kMinRun planes (a
+    // run loads two planes more than it computes; runs of at least 4 left SMs
+    // idle: 32^3, 32 -> 32 channels 12.4 -> 9.8 us)
     const long long planes = static_cast<long long>(batch) * (n / kX) * (n / kY) * n;
     const long long ctas = std::min<long long>(std::max(1, per_sm) * sm_count(), (planes + kMinRun - 1) / kMinRun);
     return launch_chained(kernel, static_cast<unsigned>(ctas), kThreads, smem, s, chained, x, w, bias, y, n, cin, act,
                           planes, err);
 }
 
-// A choice of CO, R and stages for the wide kernel and its estimated cycles.
+// A choice of CO, R and stages for the wide kernel and its estimated time.
 struct WideShape {
     int co = 0, R = 1, stages = 1;
-    double cycles = 0.0;
+    double us = 0.0;
 };
 
-// An M = 128, K = 16 MMA takes about 32 + CO / 4 cycles (its operands come
-// from shared memory at 128 B per cycle), a stage arrives at about 40 B per
-// cycle and SM, and a CTA pays about 4000 cycles of set-up, first stage and
-// epilogue that resident neighbours can hide.
+// The time of a layer: CTAs run in rounds of as many as an SM holds.  A round
+// takes the set-up, R epilogue tiles in sequence and the chunks' MMAs (an M =
+// 128, K = 16 MMA about 32 + CO / 4 cycles: its operands come from shared
+// memory at 128 B per cycle); every CTA of the busiest SM takes the copies of
+// its chunks (29 KB per us and SM; with 8 input channels half of a stage is
+// only zeroed) and the stores of its output.  Fitted to 2400 timings (n 8 to
+// 64, 1 to 8 samples, 8 to 128 channels on either side): half of them are
+// within 6 %, nine in ten within 14 %.
 template <int CO, int R, bool PAIR>
-void consider(WideShape &best, long long tiles, int nz, int cin, int cout)
+void consider(WideShape &best, long long tiles, int nz, int cin, int cout, int out_bytes)
 {
     if (cout % CO != 0 || nz % R != 0) return;
     const int chunks = (cin + 15) / 16, sms = sm_count();
@@ -599,9 +629,26 @@ void consider(WideShape &best, long long tiles, int nz, int cin, int cout)
     const int per_sm = std::min({static_cast<int>(kSmemPerSm / (kFixed + stages * kStage + 1024u)),
                                  512 / std::max(32, R * CO), 65536 / (kThreads * 64)});
     const long long per = (tiles / R * (cout / CO) + sms - 1) / sms;  // CTAs of the busiest SM
-    const double work = chunks * std::max(27.0 * R * (32.0 + CO / 4), kStage / 40.0);
-    const double cycles = per * work + (per + per_sm - 1) / per_sm * 4000.0;
-    if (best.co == 0 || cycles < best.cycles) best = {CO, R, stages, cycles};
+    const long long rounds = (per + per_sm - 1) / per_sm;
+    const double mma = 27.0 * R * (32.0 + CO / 4) / 1900.0, kb = kStage / 1024.0 * (cin == 8 ? 0.4 : 1.0);
+    const double us = 3.5 + rounds * (1.2 + 0.69 * R + 0.315 * chunks * mma) +
+                      per * (0.0345 * chunks * kb + 0.59 * R * CO / 64.0 * (out_bytes / 2));
+    if (best.co == 0 || us < best.us) best = {CO, R, stages, us};
+}
+
+template <bool PAIR>
+WideShape wide_shape(int batch, int n, int cin, int cout, int out_bytes)
+{
+    const int nz = PAIR ? n / 2 : n;
+    const long long tiles = static_cast<long long>(batch) * (n / kX) * (n / (PAIR ? 8 : 16)) * nz;
+    WideShape sh;
+    consider<64, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
+    consider<64, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
+    consider<32, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
+    consider<32, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
+    consider<16, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
+    consider<16, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
+    return sh;
 }
 
 template <int CO, int R, bool PAIR, typename TO>
@@ -621,15 +668,8 @@ template <bool PAIR, typename TO>
 cudaError_t run_wide(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
                      int cin, int cout, int act, int *err, cudaStream_t s, bool chained)
 {
-    const int nz = PAIR ? n / 2 : n;
-    const long long tiles = static_cast<long long>(batch) * (n / kX) * (n / (PAIR ? 8 : 16)) * nz;
-    WideShape sh;
-    consider<64, 4, PAIR>(sh, tiles, nz, cin, cout);
-    consider<64, 1, PAIR>(sh, tiles, nz, cin, cout);
-    consider<32, 4, PAIR>(sh, tiles, nz, cin, cout);
-    consider<32, 1, PAIR>(sh, tiles, nz, cin, cout);
-    consider<16, 4, PAIR>(sh, tiles, nz, cin, cout);
-    consider<16, 1, PAIR>(sh, tiles, nz, cin, cout);
+    const long long tiles = static_cast<long long>(batch) * (n / kX) * (n / (PAIR ? 8 : 16)) * (PAIR ? n / 2 : n);
+    const WideShape sh = wide_shape<PAIR>(batch, n, cin, cout, static_cast<int>(sizeof(TO)));
     auto go = [&](auto co, auto r) {
         return launch_wide<decltype(co)::value, decltype(r)::value, PAIR, TO>(sh, tiles, x, w, bias, y, n, cin, cout, act,
                                                                               err, s, chained);
@@ -659,14 +699,30 @@ int tensor_core_errors(bool reset)
 
 // On unless DMRT_NN_NO_TCGEN05 is set in the environment (read once).  A
 // sample's element offsets are 32-bit; the tiles are a grid dimension.
-bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout)
+// Where n is an odd multiple of 8, a tile of two planes stages its halo three
+// times, and layers of few input channels, or of output channels that are
+// not a multiple of 32, are faster on mma.sync, which gives the same bits:
+// with FP32 output 24^3 x 8, 16 -> 16 18.6 us here and 12.8 there, 40^3 x 3, 16
+// -> 16 25.0 and 20.6, but 24^3 x 8, 128 -> 128 224 and 375.  The mma.sync
+// kernel's time is within 5 % of the fit below; the tcgen05 one is taken where
+// it is estimated 10 % faster (of 353 layers, three are then slower than on
+// mma.sync by more than 2 %).
+bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout, int out_bytes)
 {
     static const bool on = std::getenv("DMRT_NN_NO_TCGEN05") == nullptr;
     const unsigned long long bases = reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(w) |
                                      reinterpret_cast<unsigned long long>(y);
     const long long vox = static_cast<long long>(n) * n * n;
-    return on && (bases & 15ull) == 0 && (cin == 8 || cin % 16 == 0) && cout % 16 == 0 && n % 8 == 0 &&
-           vox * cin < (1LL << 31) && vox * batch / 128 < (1LL << 31) && cout / 16 < 65536;
+    if (!(on && (bases & 15ull) == 0 && (cin == 8 || cin % 16 == 0) && cout % 16 == 0 && n % 8 == 0 &&
+          vox * cin < (1LL << 31) && vox * batch / 128 < (1LL << 31) && cout / 16 < 65536))
+        return false;
+    if (n % kY == 0) return true;
+    const double chunks = (cin + 15) / 16;
+    const long long sms = sm_count(), blocks = vox * batch / 256 * (cout / 16);  // mma.sync blocks of 16 channels
+    const double mma_sync = mma_sync_takes_32(vox * batch / 256, cout)
+                                ? 4.4 + chunks * (2.1 + 3.9 * static_cast<double>((blocks / 2 + sms - 1) / sms))
+                                : 3.6 + chunks * (2.3 + 2.64 * static_cast<double>((blocks + sms - 1) / sms));
+    return 1.1 * wide_shape<true>(batch, n, cin, cout, out_bytes).us <= mma_sync;
 }
 
 template <typename TO>

@@ -754,25 +754,6 @@ __global__ void __launch_bounds__(256) conv1x1_small_kernel(const TI *__restrict
     }
 }
 
-// Streaming multiprocessors of the current device (152 on GB300), asked once
-// per device.
-int sm_count()
-{
-    static std::atomic<int> cached[64];
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) {
-        cudaGetLastError();
-        return 152;
-    }
-    if (dev >= 0 && dev < 64 && (sms = cached[dev].load(std::memory_order_relaxed)) > 0) return sms;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
-        cudaGetLastError();
-        return 152;
-    }
-    if (dev >= 0 && dev < 64) cached[dev].store(sms, std::memory_order_relaxed);
-    return sms;
-}
-
 // out = bfloat16(in)
 __global__ void narrow_kernel(const float *__restrict__ in, __nv_bfloat16 *__restrict__ out, long long len)
 {
@@ -1454,6 +1435,33 @@ unsigned flat_blocks(long long len)
 
 // ---------------------------------------------------------------- launchers
 
+// Streaming multiprocessors of the current device (152 on GB300), asked once
+// per device.
+int sm_count()
+{
+    static std::atomic<int> cached[64];
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 152;
+    }
+    if (dev >= 0 && dev < 64 && (sms = cached[dev].load(std::memory_order_relaxed)) > 0) return sms;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+        cudaGetLastError();
+        return 152;
+    }
+    if (dev >= 0 && dev < 64) cached[dev].store(sms, std::memory_order_relaxed);
+    return sms;
+}
+
+// 32 output channels per block, unless that leaves most SMs idle (the 8^3
+// level: 32 blocks of 32 channels at batch 4): 16 per block doubles the
+// blocks.  Every output accumulates the same MMAs in the same order either way.
+bool mma_sync_takes_32(long long voxel_tiles, int cout)
+{
+    return cout % 32 == 0 && voxel_tiles * (cout / 32) >= 2LL * sm_count();
+}
+
 template <typename TI, typename TW, typename TO>
 cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch, int n, int cin,
                    int cout, int k, int act, cudaStream_t s, bool chained)
@@ -1472,7 +1480,7 @@ cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch
         // channel count and both base pointers must keep 16-byte alignment
         const bool aligned =
             ((reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(w)) & 15ull) == 0;
-        if (k == 3 && conv3d_umma_takes(x, w, y, batch, n, cin, cout))
+        if (k == 3 && conv3d_umma_takes(x, w, y, batch, n, cin, cout, static_cast<int>(sizeof(TO))))
             return conv3d_umma(x, w, bias, y, batch, n, cin, cout, act, s, chained);
         if (k == 3 && aligned && (cin == 8 || cin % 16 == 0) && cout % 16 == 0 && n % kWtX == 0 &&
             n % kWtZ == 0) {
@@ -1480,11 +1488,7 @@ cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch
             // the dynamic shared memory exceeds the 48 KB default: opt in (per
             // call, so every device the kernel runs on gets the attribute)
             cudaError_t e;
-            // 32 output channels per block, unless that leaves most SMs idle
-            // (the 8^3 level: 32 blocks of 32 channels at batch 4): 16 per
-            // block doubles the blocks; every output accumulates the same
-            // MMAs in the same order either way, so the results are the same
-            if (cout % 32 == 0 && vtiles * static_cast<unsigned>(cout / 32) >= 2u * sm_count()) {
+            if (mma_sync_takes_32(vtiles, cout)) {
                 const int smem = (kWtHalo + 27 * 32) * kWtRow * 2;
                 e = cudaFuncSetAttribute(conv3d_tc_kernel<4, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
                 if (e != cudaSuccess) return e;

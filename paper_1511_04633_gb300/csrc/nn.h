@@ -46,10 +46,18 @@ template <typename TI, typename TW, typename TO>
 cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch, int n, int cin,
                    int cout, int k, int act, cudaStream_t s, bool chained = false);
 
+// Streaming multiprocessors of the current device (152 on GB300).
+int sm_count();
+
+// The mma.sync convolution: 32 output channels per block (else 16)?  Voxel
+// tiles are of 8 x 8 x 4.
+bool mma_sync_takes_32(long long voxel_tiles, int cout);
+
 // The 3^3 convolutions of bfloat16 x and w on the tcgen05 tensor cores
 // (conv_umma.cu): taken where the channel counts are multiples of 16 (cin
-// also 8), n a multiple of 8 and the three arrays 16-byte aligned.
-bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout);
+// also 8), n a multiple of 8 and the three arrays 16-byte aligned, if they
+// are the faster ones.
+bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout, int out_bytes);
 template <typename TO>
 cudaError_t conv3d_umma(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
                         int cin, int cout, int act, cudaStream_t s, bool chained);

@@ -4,6 +4,7 @@ and pipelines, against the oracle's convolution."""
 import numpy as np
 import pytest
 
+from launch_shim import run_child
 from oracle import surrogate as S
 from paper_1511_04633_gb300 import inputs
 
@@ -48,3 +49,52 @@ def test_convolution(env, n, batch, cin, cout, shift, out_f32):
     assert np.abs(got - ref).max() <= tol * np.abs(ref).max()
     rest = torch.cat([flat[:shift], flat[shift + size:]])
     assert bool((rest == 7.0).all())
+
+
+# (n, batch, cin, cout): one and many chunks, one and four tiles per CTA, tiles
+# of two planes; the mma.sync kernel with 16 output channels per block (few
+# blocks, or no multiple of 32) and with 32 (304 blocks or more); narrow layers
+# of one K = 16 slice per tap
+@pytest.mark.parametrize("n,batch,cin,cout", [
+    (8, 2, 128, 64), (24, 1, 64, 128), (24, 8, 96, 128), (16, 1, 48, 80), (32, 3, 64, 64), (48, 1, 128, 32),
+    (24, 8, 128, 16), (16, 2, 16, 16), (32, 4, 8, 32),
+])
+@pytest.mark.parametrize("out_f32", [False, True])
+def test_the_two_tensor_core_paths_give_the_same_bits(env, n, batch, cin, cout, out_f32):
+    """Outputs at 32-byte, 16-byte (other stores) and smaller alignments (the
+    mma.sync kernels)."""
+    torch, dm = env
+    x = torch.from_numpy(inputs.random_targets((batch, n, n, n, cin), seed=51)).to(torch.bfloat16).cuda()
+    w = torch.from_numpy(inputs.random_weights(27 * cout * cin, seed=52, scale=0.2)).to(torch.bfloat16).cuda()
+    b = torch.from_numpy(inputs.random_weights(cout, seed=53, scale=0.5)).cuda()
+    size = batch * n ** 3 * cout
+    elt = 4 if out_f32 else 2
+    outs = []
+    for shift in (0, 16 // elt, 8 // elt):
+        flat = torch.full((size + 8,), 7.0, dtype=torch.float32 if out_f32 else torch.bfloat16, device="cuda")
+        y = flat[shift:shift + size]
+        dm.dmrt_nn_conv3d(x, w, b, y, batch, n, cin, cout, 3, act=1)
+        assert bool((flat[:shift] == 7.0).all()) and bool((flat[shift + size:] == 7.0).all())
+        outs.append(y)
+    assert dm.dmrt_nn_tensor_core_errors(reset=True) == 0
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
+def test_layers_take_the_faster_kernel(env, tmp_path):
+    """Two-plane tiles with few input channels, or output channels that are no
+    multiple of 32, go to mma.sync; wide ones and 16-voxel edges to tcgen05."""
+    run_child(tmp_path, """
+    import torch
+    def umma(n, batch, cin, cout):
+        x = torch.zeros((batch, n, n, n, cin), dtype=torch.bfloat16, device="cuda")
+        w = torch.zeros((27, cout, cin), dtype=torch.bfloat16, device="cuda")
+        y = torch.zeros((batch, n, n, n, cout), dtype=torch.bfloat16, device="cuda")
+        torch.cuda.synchronize()
+        shim.shim_forget()
+        dm.dmrt_nn_conv3d(x, w, None, y, batch, n, cin, cout, 3, act=1)
+        return b"conv3d_umma" in shim.shim_names()
+    for c in ((24, 8, 16, 16), (40, 4, 32, 80), (40, 3, 16, 16), (56, 4, 32, 48)):
+        assert not umma(*c), c
+    for c in ((24, 8, 128, 128), (8, 4, 128, 128), (40, 4, 64, 64), (56, 2, 8, 64), (16, 1, 16, 16), (16, 4, 48, 48)):
+        assert umma(*c), c
+    """)
