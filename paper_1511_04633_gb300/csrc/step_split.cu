@@ -13,12 +13,8 @@
 // 61 in place FP16 14.8 -> 11.4 us, two buffers BF16 13.6 -> 11.3, FP32 15.4
 // -> 13.3; 255^3 BF16 419 -> 377 us (in place 404 -> 357), FP32 559 -> 557.
 // It executes half the instructions but holds half the warps for the same
-// cells, so it pays where those fill the SMs: from 300,000 cells (69^3 BF16
-// 11.8 -> 8.6 us), and below that, down to 60,000, where one round of
-// resident blocks covers the box (39^3 BF16 4.6 -> 3.5 us; 55^3 5.8 -> 5.4;
-// the worst case in that range, 49^3, loses 0.3 us of 5.0 with two buffers).
-// With a second, nearly empty round (61^3) it was no faster (7.0 against 6.8
-// us), nor below (31^3: 2.8 against 2.5 us).
+// cells, so it pays where those fill the SMs (step_split_pays): 69^3 BF16 11.8
+// -> 8.6 us, 45^3 4.7 -> 3.9, but 47^3 4.7 -> 5.2.
 //
 // A slab's cells are numbered flat (c = y nx + x), 128 per block, so no lane
 // idles at the end of a row; y = c / nx is a multiplication (RowDivisor).
@@ -278,10 +274,29 @@ bool step_split_supported(int wall, const Geometry &G)
     return wall >= 1 && wall <= 3 && static_cast<long long>(G.nx) * G.ny < (1LL << 28) - kSplitThreads;
 }
 
+// For small boxes both kernels' times are steps of their blocks per SM (152).
+// Two buffers, FP32 and 16-bit, us per step: one cell per thread 2.5 to 3.4 for
+// up to 3 blocks, 4.1 to 5.1 for 4 to 7, 4.6 to 6.4 for 8 to 10, 5.6 to 7.4 for
+// 11 and 12; this kernel 2.5 to 2.8 for 1, 2.8 to 4.2 for 2, 3.7 to 4.6 up to
+// 2.5, 4.8 to 6.1 up to 5 (the hardware spreads more than 380 blocks
+// unevenly), 5.7 to 7.3 for 6.  Each row of the table: up to so many blocks of
+// this kernel, it is taken from so many one-cell blocks on; beyond it, from 1.8
+// times its own (thin boxes pair a slab with none).  Of 190 boxes of 25,000 to
+// 2,000,000 cells, in six variants each, 15 of 1140 are slower than on the
+// one-cell kernels by more than 1.5 % (three by 5 to 11 %), 14 would gain 3 %
+// or more here; a line at 60,000 cells and one round of blocks made 84 slower,
+// by up to 30 % (165 x 11 x 55 FP32 4.6 -> 6.0 us).  Boxes below 60,000 cells,
+// or of more than one round of blocks below 300,000, stay on the one-cell kernels.
 bool step_split_pays(const Geometry &G)
 {
     const long long cells = static_cast<long long>(G.nx) * G.ny * G.nz;
-    return cells >= 300000 || (cells >= 60000 && split_blocks(G) <= 152 * kSplitBlocks);
+    const long long blocks = static_cast<long long>(split_blocks(G));
+    if (cells < 300000 && (cells < 60000 || blocks > 152 * kSplitBlocks)) return false;
+    const long long one_cell = static_cast<long long>((G.nx + 31) / 32) * ((G.ny + 3) / 4) * G.nz;
+    constexpr int kLine[][2] = {{152, 456}, {290, 555}, {304, 608}, {380, 684}, {760, 1368}};
+    for (const auto &l : kLine)
+        if (blocks <= l[0]) return one_cell >= l[1];
+    return 5 * one_cell >= 9 * blocks;
 }
 
 size_t split_blocks(const Geometry &G)

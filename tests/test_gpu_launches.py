@@ -123,3 +123,20 @@ def test_autotune_times_the_kernels_that_step(tmp_path, each, storage, twos):
     for k in range(len(cav)):
         assert np.array_equal(a.populations(k)[0], ref.populations(k)[0])
     """)
+
+
+@pytest.mark.parametrize("grid,split", [
+    ((47, 47, 47), False), ((49, 49, 49), False), ((165, 11, 55), False), ((217, 183, 3), False), ((39, 39, 39), False),
+    ((45, 45, 45), True), ((55, 55, 55), True), ((33, 1000, 2), True), ((69, 69, 69), True), ((101, 75, 61), True),
+])
+@pytest.mark.parametrize("streaming", [0, 1])
+def test_boxes_with_odd_rows_take_the_faster_kernel(tmp_path, grid, split, streaming):
+    """By the blocks that either kernel would have per SM."""
+    run_child(tmp_path, f"""
+    for storage in (0, 1, 2):
+        cav = dm.Cavity({grid}, 1e4, wall_type=1, storage=storage, streaming={streaming}, residual_interval=20)
+        shim.shim_forget()
+        cav.step(4)
+        names = shim.shim_names().decode().split()
+        assert names and all(("split" in n) == {split} for n in names), names
+    """)

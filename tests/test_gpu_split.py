@@ -50,3 +50,17 @@ def test_bitwise_the_one_cell_kernels(dm, grid, wall, storage, streaming, roundi
     assert abs(a.residual() - b.residual()) <= 1e-12 * b.residual()
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("streaming", [0, 1])
+def test_two_slabs_bitwise_the_one_cell_kernels(dm, streaming):
+    a = _cavity(dm, (33, 1000, 2), 3, 1, streaming, 0)
+    b = _cavity(dm, (33, 1000, 2), 3, 1, streaming, 1)
+    for n in (1, 4, 15, 2):
+        a.step(n)
+        b.step(n)
+        for p, q in zip(a.populations(), b.populations()):
+            assert np.array_equal(p, q)
+    assert abs(a.residual() - b.residual()) <= 1e-12 * b.residual()
+    a.close()
+    b.close()
