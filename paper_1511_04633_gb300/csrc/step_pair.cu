@@ -468,7 +468,12 @@ int tile_width(int row, int &slots)
 //   in place     BF16 70^3 9.7 -> 7.3, 112^3 26.0 -> 23.4; but 190 x 126 x 90
 //     (1 % idle) 36.7 -> 40.2, FP32 60^3 (6 %) 6.08 -> 6.22
 // Boxes of 2.5 to 4 flat blocks per SM keep the tiles: FP32 48^3 4.5 -> 5.0
-// us, 52^3 4.7 -> 4.9; so do the smallest in place (16^3: 1.94 -> 2.07).
+// us, 52^3 4.7 -> 4.9; so do the smallest in place (16^3: 1.94 -> 2.07), and
+// boxes just beyond either line whose tiles are few as well: 54^3 in place FP32
+// 4.75 -> 5.21, 108 x 77 x 19 FP32 4.56 -> 4.89, 28 x 46 x 24 in place FP16 2.38 -> 2.59
+// (but with tiles of 16 pairs 206 x 8 x 96 FP16 5.05 -> 4.30, and 84 x 96 x 4 in place
+// 2.55 -> 2.34).  Of 1848 timed cases, five of the flat ones are then slower than
+// their tiles by 2 % or more (3 % at most).
 // A step that takes a residual point always uses the row tiles: the order of
 // its sums, and so the residual, is then the same in either scheme.
 bool pair_flat(const Geometry &G, bool inplace, bool res)
@@ -479,6 +484,10 @@ bool pair_flat(const Geometry &G, bool inplace, bool res)
     const long long pairs = static_cast<long long>(row) * G.ny * G.nz;
     const long long blocks = (pairs + kPairThreads - 1) / kPairThreads;
     if ((blocks > 380 && blocks <= 610) || (inplace && blocks <= 100)) return false;
+    // the tiles fill one round (or one block per SM) just as well
+    const long long tiles = static_cast<long long>((row + bx - 1) / bx) * ((G.ny + by - 1) / by) * G.nz;
+    if (blocks > 610 && blocks <= 640 && bx > 16 && tiles <= 152 * kPairBlocks) return false;
+    if (inplace && blocks <= 125 && tiles <= 152) return false;
     const double idle = 1.0 - static_cast<double>(row) * G.ny / (static_cast<double>(slots) * ((G.ny + by - 1) / by * by));
     return inplace ? idle > 0.08 : idle > 0.03 || G.nx % 32 != 0;
 }
