@@ -618,10 +618,10 @@ struct WideShape {
 // 64, 1 to 8 samples, 8 to 128 channels on either side): half of them are
 // within 6 %, nine in ten within 14 %.
 template <int CO, int R, bool PAIR>
-void consider(WideShape &best, long long tiles, int nz, int cin, int cout, int out_bytes)
+void consider(WideShape &best, long long tiles, int nz, int cin, int cout, int out_bytes, int sms)
 {
     if (cout % CO != 0 || nz % R != 0) return;
-    const int chunks = (cin + 15) / 16, sms = sm_count();
+    const int chunks = (cin + 15) / 16;
     constexpr unsigned kFixed = kHead + table_bytes<PAIR>(R), kStage = stage_bytes<CO, PAIR>(R);
     int stages = std::min(chunks, kMaxStages);
     while (stages > 1 && kFixed + stages * kStage > kSmemPerCta) --stages;
@@ -641,13 +641,14 @@ WideShape wide_shape(int batch, int n, int cin, int cout, int out_bytes)
 {
     const int nz = PAIR ? n / 2 : n;
     const long long tiles = static_cast<long long>(batch) * (n / kX) * (n / (PAIR ? 8 : 16)) * nz;
+    const int sms = sm_count();
     WideShape sh;
-    consider<64, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
-    consider<64, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
-    consider<32, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
-    consider<32, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
-    consider<16, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
-    consider<16, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes);
+    consider<64, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
+    consider<64, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
+    consider<32, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
+    consider<32, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
+    consider<16, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
+    consider<16, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
     return sh;
 }
 
