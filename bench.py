@@ -73,6 +73,15 @@ KERNEL_SOURCES = {"ab": ["paper_1511_04633_gb300/csrc/step.cu"] + _BODY,
                   "inplace_pair": ["paper_1511_04633_gb300/csrc/step_pair.cu",
                                    "paper_1511_04633_gb300/csrc/pair_body.cuh"] + _BODY}
 STEP_KERNEL_SOURCES = KERNEL_SOURCES["ab"]
+SCHEMES = {"step_kernel": "ab", "step_pair_kernel": "pair", "step_pair_tma_kernel": "pair_tma",
+           "step_inplace_kernel": "inplace", "step_inplace_pair_kernel": "inplace_pair"}
+
+
+def kernel_label(name: str, wall: int, storage: str) -> str:
+    """dmrt_step_kernel's name with the wall type and storage of the run."""
+    base, _, twos = name.partition(" ")
+    both = (" (both phases, by twos)" if twos else " (both phases)") if "inplace" in base else ""
+    return f"{base}<{wall}, {storage}>{both}"
 
 
 # ---------------------------------------------------------------- distributed plumbing
@@ -192,7 +201,10 @@ def step_kernel_digest(scheme: str = "ab") -> str:
 def profiled_traffic(storage: str = "f32", wall: int = 2, scheme: str = "ab"):
     """DRAM bytes per step-kernel launch from the committed ncu summary, only
     if it was taken on the current kernel sources for this storage, wall and
-    kernel scheme ("ab", "pair", "pair_tma", "inplace" or "inplace_pair")."""
+    kernel scheme ("ab", "pair", "pair_tma", "inplace" or "inplace_pair";
+    None, a kernel without a summary, has no figure)."""
+    if scheme is None:
+        return None
     path = os.path.join(ROOT, "profiles", "step_kernel_traffic.json")
     try:
         with open(path) as fh:
@@ -288,10 +300,7 @@ def run_dmrt(args, rank, local, world):
     dmrt.dmrt_set_stream(cav.h, stream)
     inner = args.inner
     cpt = cav.params["cells_per_thread"]
-    if args.streaming == "inplace":
-        scheme = {1: "inplace", 2: "inplace_pair"}[cpt]
-    else:
-        scheme = {1: "ab", 2: ("pair_tma" if cav.params["pair_loads"] == 2 else "pair")}[cpt]
+    kernel = cav.step_kernel
 
     def one_step():
         dmrt.dmrt_step(cav.h, inner)
@@ -327,7 +336,7 @@ def run_dmrt(args, rank, local, world):
     bytes_per_cell = stats["bytes_per_cell"]
     achieved = bytes_per_cell * cells / launch_s / 1e9
     peak, peak_src = measured_peaks()
-    traffic = profiled_traffic(args.storage, args.wall, scheme)
+    traffic = profiled_traffic(args.storage, args.wall, SCHEMES.get(kernel))
 
     # end to end through the C ABI with host buffers: upload the start fields
     # from pinned memory, step, read the fields and Nu back
@@ -394,13 +403,7 @@ def run_dmrt(args, rank, local, world):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
                      "nominal_peak": NOMINAL_HBM_GBS, "frac_nominal": achieved / NOMINAL_HBM_GBS,
-                     "kernel": {"ab": f"step_kernel<{args.wall}, {args.storage}>",
-                                "pair": f"step_pair_kernel<{args.wall}, {args.storage}>",
-                                "pair_tma": f"step_pair_tma_kernel<{args.wall}, {args.storage}>",
-                                "inplace": f"step_inplace_kernel<{args.wall}, {args.storage}> "
-                                           "(both phases)",
-                                "inplace_pair": f"step_inplace_pair_kernel<{args.wall}, {args.storage}> "
-                                                "(both phases)"}[scheme],
+                     "kernel": kernel_label(kernel, args.wall, args.storage),
                      "bytes_per_cell": bytes_per_cell, "launch_us": launch_s * 1e6},
         "cpu_baseline": cpu,
         "e2e": {"value": e2e_value, "unit": "MLUPS", "h2d_bytes_per_step": h2d,
@@ -505,10 +508,9 @@ def measure_ensemble(dmrt, inputs, torch, stream, gpu, *, members, seed, storage
     draws = inputs.ensemble_draws(members, seed=seed)
     cav = [{"grid": (d["n"],) * 3, "Ra": d["Ra"], "wall": d["wall"]} for d in draws]
     ens = dmrt.Ensemble(cav, storage=storage, streaming=streaming)
-    ens_kernel = ("ensemble_pair_kernel" if ens.params(0)["cells_per_thread"] == 2
-                  else "ensemble_step_kernel") + (" (in place, both phases)" if streaming else "")
     dmrt.dmrt_ensemble_set_stream(ens.e, stream)
     report = ens.autotune(trials=3)
+    ens_kernel = ens.step_kernel
     cells = ens.cells
 
     def one_step():
@@ -605,11 +607,10 @@ def measure_cavity(dmrt, torch, stream, gpu, *, grid, wall, ra, storage, inner, 
     launch_s = stats["step_ms"] / 1e3 / max(stats["timed_steps"], 1)
     achieved = stats["bytes_per_cell"] * cells / launch_s / 1e9
     peak, peak_src = measured_peaks()
-    params = cav.params
+    kernel = cav.step_kernel
     cav.close()
     names = {v: k for k, v in STORAGES.items()}
-    kernel = "step_pair_kernel" if params["cells_per_thread"] == 2 else "step_kernel"
-    traffic = profiled_traffic(names[storage], wall, "pair" if params["cells_per_thread"] == 2 else "ab")
+    traffic = profiled_traffic(names[storage], wall, SCHEMES.get(kernel))
     return {
         "value": cells * inner * steps / secs / 1e6, "unit": "MLUPS", "steps": steps, "warmup": warmup,
         "ms_per_step": secs / steps * 1e3,
@@ -619,7 +620,7 @@ def measure_cavity(dmrt, torch, stream, gpu, *, grid, wall, ra, storage, inner, 
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
                      "nominal_peak": NOMINAL_HBM_GBS, "frac_nominal": achieved / NOMINAL_HBM_GBS,
-                     "kernel": f"{kernel}<{wall}, {names[storage]}>", "bytes_per_cell": stats["bytes_per_cell"],
+                     "kernel": kernel_label(kernel, wall, names[storage]), "bytes_per_cell": stats["bytes_per_cell"],
                      "launch_us": launch_s * 1e6},
         "gpu_launches": stats["total_launches"], "clocks": clocks.summary(),
     }

@@ -81,9 +81,11 @@ typedef enum {
 /* How the populations stream (the method is the same; only the memory
  * scheme differs).
  *  AB     : two population buffers; each step pulls from one and writes the
- *           other (2 x 26 values per cell held on the device).  Sizes whose
- *           working set then fits L2 (and 16-bit ensembles) take plain steps
- *           two at a time within one buffer; the values are the same.
+ *           other (2 x 26 values per cell held on the device).  Where that is
+ *           faster, plain steps run two at a time within one buffer, with
+ *           the same values (dmrt_step_kernel): cavities whose buffer has 45
+ *           to 117 MB (with odd nx also larger ones), ensembles stepped by
+ *           shape groups from 45 MB per buffer (FP32 up to 110 MB).
  *  INPLACE: one buffer updated in place by two alternating kernels (the AA
  *           access pattern): half the population memory, the same HBM
  *           traffic per step, and bitwise the same results as AB in every
@@ -297,6 +299,12 @@ dmrt_status dmrt_set_diffusion(dmrt_t *h, const double D[9]);
 /* Read the derived lattice parameters. */
 dmrt_status dmrt_get_params(const dmrt_t *h, dmrt_params *out);
 
+/* The name of the kernel that plain steps (those that take no residual
+ * point) run: which of the equivalent step kernels the box's size, storage and
+ * options select.  " by twos" after the name of an in-place kernel: a
+ * two-buffer state takes its steps in pairs within one buffer.  "" for NULL. */
+const char *dmrt_step_kernel(const dmrt_t *h);
+
 /* Enable (1) or disable (0) CUDA-event timing of the step kernels. */
 dmrt_status dmrt_set_timing(dmrt_t *h, int enabled);
 
@@ -388,6 +396,9 @@ dmrt_status dmrt_ensemble_get_populations(dmrt_ensemble_t *e, int member, float 
 dmrt_status dmrt_ensemble_member_params(const dmrt_ensemble_t *e, int member, dmrt_params *out);
 
 /* Text of the last error on this ensemble ("" if none). */
+/* As dmrt_step_kernel, for an ensemble. */
+const char *dmrt_ensemble_step_kernel(const dmrt_ensemble_t *e);
+
 const char *dmrt_ensemble_last_error(const dmrt_ensemble_t *e);
 
 /* ------------------------------------------------------------------------

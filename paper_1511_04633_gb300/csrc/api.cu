@@ -997,6 +997,17 @@ dmrt_status dmrt_get_params(const dmrt_t *h, dmrt_params *out)
     return DMRT_OK;
 }
 
+const char *dmrt_step_kernel(const dmrt_t *h)
+{
+    if (!h) return "";
+    const bool pairs = h->cells_per_thread == 2;
+    // (a pair of in-place steps never includes the last two of an interval)
+    if (h->ab_inplace && h->K > 2) return pairs ? "step_inplace_pair_kernel by twos" : "step_inplace_split_kernel by twos";
+    if (h->inplace) return h->split ? "step_inplace_split_kernel" : pairs ? "step_inplace_pair_kernel" : "step_inplace_kernel";
+    if (h->split) return "step_split_kernel";
+    return !pairs ? "step_kernel" : h->pair_loads == 2 ? "step_pair_tma_kernel" : "step_pair_kernel";
+}
+
 dmrt_status dmrt_set_diffusion(dmrt_t *h, const double D[9])
 {
     if (!h || !D) return DMRT_ERR_ARG;

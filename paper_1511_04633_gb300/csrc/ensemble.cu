@@ -2194,6 +2194,17 @@ dmrt_status dmrt_ensemble_member_params(const dmrt_ensemble_t *e, int member, dm
     return DMRT_OK;
 }
 
+const char *dmrt_ensemble_step_kernel(const dmrt_ensemble_t *e)
+{
+    if (!e) return "";
+    if (e->grouped) {
+        if (e->by_twos && e->K > 2) return "ensemble_group_inplace_pair_kernel by twos";
+        return e->inplace ? "ensemble_group_inplace_pair_kernel" : "ensemble_group_pair_kernel";
+    }
+    if (e->pairs) return e->inplace ? "ensemble_inplace_pair_kernel" : "ensemble_pair_kernel";
+    return e->inplace ? "ensemble_inplace_kernel" : "ensemble_step_kernel";
+}
+
 const char *dmrt_ensemble_last_error(const dmrt_ensemble_t *e)
 {
     if (!e) return "null ensemble";

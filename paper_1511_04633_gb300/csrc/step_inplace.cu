@@ -189,14 +189,17 @@ void fill_ab_inplace_geometry(const Geometry &G, InplaceGeometry &SI)
     }
 }
 
-// In place, the state is one buffer instead of two: a cavity whose one buffer
-// stays in L2 (129 MB) while two do not steps faster.  Measured on GB300, per
-// step, two buffers -> in place: FP32 80^3 13.3 -> 10.8 us, 96^3 28.2 ->
-// 21.5; 16-bit 96^3 15.7 -> 15.2, 112^3 28.4 -> 23.4, 190 x 126 x 90 41.6 ->
-// 36.7, 128^3 39.5 -> 39.0; below and above (FP32 60^3 5.8 -> 6.1, 112^3 44.1
-// -> 44.9, BF16 142^3 54.6 -> 55.3) two buffers are as fast or faster.  With
-// odd rows (split) the stores between buffers share sectors at every row end
-// and in place stays faster: 127^3 BF16 47.3 -> 42.0, 255^3 375 -> 357 us.
+// In place, the state is one buffer instead of two and stays in L2 (129 MB) up
+// to twice the size.  The lines: from 90 MB of two buffers, of which L2 then
+// keeps too little from one step to the next, up to 117 MB of one.  Measured
+// on GB300, per step, two buffers -> in place: FP32 80^3 13.3 -> 10.8 us, 96^3
+// 28.2 -> 21.5, 160 x 28 x 250 (116 MB) 36.6 -> 34.5; 16-bit 96^3 15.7 -> 15.2,
+// 112^3 28.4 -> 23.4, 190 x 126 x 90 41.6 -> 36.7, 128^3 39.5 -> 39.0; below and
+// above (FP32 60^3 5.8 -> 6.1, 112^3 (146 MB) 44.1 -> 44.9, BF16 142^3 (149 MB)
+// 54.6 -> 55.3) two buffers are as fast or faster; between 117 and 146 MB
+// nothing was measured.  With odd rows (split) the stores between buffers
+// share sectors at every row end and in place stays faster at any size: 127^3
+// BF16 47.3 -> 42.0, 255^3 375 -> 357 us (117 x 40 x 261 FP32 loses 2.6 %).
 bool inplace_pays(const Geometry &G, int storage, bool split)
 {
     const long long bytes = static_cast<long long>(G.plane) * kPlanes * storage_bytes(storage);

@@ -112,6 +112,7 @@ def load(build_if_missing: bool = True):
             "dmrt_get_populations": ([vp, vp, vp, i], i),
             "dmrt_init_fields": ([vp, vp, vp, vp, i], i),
             "dmrt_get_params": ([vp, P(dmrt_params)], i),
+            "dmrt_step_kernel": ([vp], ctypes.c_char_p),
             "dmrt_set_diffusion": ([vp, P(d)], i),
             "dmrt_checkpoint_size": ([vp], ctypes.c_longlong),
             "dmrt_checkpoint_save": ([vp, vp, ctypes.c_longlong], i),
@@ -134,6 +135,7 @@ def load(build_if_missing: bool = True):
             "dmrt_ensemble_init_fields": ([vp, i, vp, vp, vp, i], i),
             "dmrt_ensemble_get_populations": ([vp, i, vp, vp, i], i),
             "dmrt_ensemble_member_params": ([vp, i, P(dmrt_params)], i),
+            "dmrt_ensemble_step_kernel": ([vp], ctypes.c_char_p),
             "dmrt_ensemble_last_error": ([vp], ctypes.c_char_p),
             "dmrt_surrogate_create": ([P(vp), P(dmrt_surrogate_cfg)], i),
             "dmrt_surrogate_destroy": ([vp], None),
@@ -433,6 +435,10 @@ class Cavity:
     def params(self):
         return dmrt_get_params(self.h)
 
+    @property
+    def step_kernel(self) -> str:
+        return load().dmrt_step_kernel(self.h).decode()
+
     def step(self, n=1):
         dmrt_step(self.h, n)
 
@@ -642,6 +648,10 @@ class Ensemble:
 
     def params(self, member):
         return dmrt_ensemble_member_params(self.e, member)
+
+    @property
+    def step_kernel(self) -> str:
+        return load().dmrt_ensemble_step_kernel(self.e).decode()
 
     def fields(self, member):
         nx, ny, nz = self.cavities[member]["grid"]

@@ -81,3 +81,12 @@ def test_traffic_is_dropped_when_the_kernel_changed(tmp_path, monkeypatch):
 def test_warmup_below_three_is_rejected():
     with pytest.raises(SystemExit):
         bench.main(["--warmup", "2"])
+
+
+def test_kernel_labels_and_their_traffic_scheme():
+    assert bench.kernel_label("step_pair_kernel", 2, "f32") == "step_pair_kernel<2, f32>"
+    assert bench.kernel_label("step_inplace_kernel", 1, "f16") == "step_inplace_kernel<1, f16> (both phases)"
+    twos = "step_inplace_pair_kernel by twos"
+    assert bench.kernel_label(twos, 3, "bf16") == "step_inplace_pair_kernel<3, bf16> (both phases, by twos)"
+    # no profile of another kernel stands in for it
+    assert bench.profiled_traffic("bf16", 3, bench.SCHEMES.get(twos)) is None

@@ -157,3 +157,44 @@ def test_boxes_with_even_rows_take_the_faster_numbering(tmp_path, grid, streamin
         names = shim.shim_names().decode().split()
         assert names and all("pair_kernel" in n and ("Lb{int(flat)}EEEv" in n) for n in names), names
     """)
+
+
+@pytest.mark.parametrize("grid,kw,name", [
+    ((32, 32, 32), {}, "step_pair_kernel"), ((32, 32, 32), {"cells_per_thread": 1}, "step_kernel"),
+    ((32, 32, 32), {"streaming": 1}, "step_inplace_pair_kernel"), ((31, 32, 32), {"streaming": 1}, "step_inplace_kernel"),
+    ((64, 64, 64), {"storage": 1, "pair_loads": 2}, "step_pair_tma_kernel"),
+    ((96, 96, 96), {"storage": 2}, "step_inplace_pair_kernel by twos"),
+    ((96, 96, 96), {"storage": 2, "residual_interval": 2}, "step_pair_kernel"),
+    ((101, 75, 61), {}, "step_inplace_split_kernel by twos"), ((101, 75, 61), {"storage": 1}, "step_split_kernel"),
+    ((101, 75, 61), {"streaming": 1}, "step_inplace_split_kernel"), ((130, 130, 130), {"wall_type": 0}, "step_kernel"),
+])
+def test_cavities_name_the_kernel_that_steps(tmp_path, grid, kw, name):
+    run_child(tmp_path, f"""
+    cav = dm.Cavity({grid}, 1e4, **{{"wall_type": 1, **{kw}}})
+    shim.shim_forget()
+    cav.step(6 if cav.params["residual_interval"] > 6 else 1)
+    names = shim.shim_names().decode().split()
+    base = {name!r}.split(" ")[0]
+    assert cav.step_kernel == {name!r}
+    # (mangled names carry their length)
+    assert names and all(f"{{len(base)}}{{base}}I" in n for n in names), names
+    """)
+
+
+@pytest.mark.parametrize("grids,kw,name", [
+    ([(48, 48, 48)] * 3, {}, "ensemble_group_pair_kernel"), ([(48, 48, 48)] * 3, {"streaming": 1}, "ensemble_group_inplace_pair_kernel"),
+    ([(48, 48, 48)] * 5, {}, "ensemble_group_inplace_pair_kernel by twos"),
+    ([(48, 48, 48)] * 5, {"residual_interval": 2}, "ensemble_group_pair_kernel"),
+    ([(31, 20, 20), (32, 20, 20)], {}, "ensemble_step_kernel"), ([(31, 20, 20)] * 2, {"streaming": 1}, "ensemble_inplace_kernel"),
+    ([(2 * k, 8, 8) for k in range(1, 41)], {}, "ensemble_pair_kernel"),
+])
+def test_ensembles_name_the_kernel_that_steps(tmp_path, grids, kw, name):
+    run_child(tmp_path, f"""
+    ens = dm.Ensemble([dict(grid=g, Ra=1e4, wall=1) for g in {grids}], **{kw})
+    shim.shim_forget()
+    ens.step(6 if ens.params(0)["residual_interval"] > 6 else 1)
+    names = [n for n in shim.shim_names().decode().split() if "residual" not in n]
+    base = {name!r}.split(" ")[0]
+    assert ens.step_kernel == {name!r}
+    assert names and all(f"{{len(base)}}{{base}}I" in n for n in names), names
+    """)
