@@ -603,12 +603,6 @@ cudaError_t launch_narrow(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const 
                           planes, err);
 }
 
-// A choice of CO, R and stages for the wide kernel and its estimated time.
-struct WideShape {
-    int co = 0, R = 1, stages = 1;
-    double us = 0.0;
-};
-
 // The time of a layer: CTAs run in rounds of as many as an SM holds.  A round
 // takes the set-up, R epilogue tiles in sequence and the chunks' MMAs (an M =
 // 128, K = 16 MMA about 32 + CO / 4 cycles: its operands come from shared
@@ -618,7 +612,7 @@ struct WideShape {
 // 64, 1 to 8 samples, 8 to 128 channels on either side): half of them are
 // within 6 %, nine in ten within 14 %.
 template <int CO, int R, bool PAIR>
-void consider(WideShape &best, long long tiles, int nz, int cin, int cout, int out_bytes, int sms)
+void consider(UmmaPlan &best, long long tiles, int nz, int cin, int cout, int out_bytes, int sms)
 {
     if (cout % CO != 0 || nz % R != 0) return;
     const int chunks = (cin + 15) / 16;
@@ -637,12 +631,12 @@ void consider(WideShape &best, long long tiles, int nz, int cin, int cout, int o
 }
 
 template <bool PAIR>
-WideShape wide_shape(int batch, int n, int cin, int cout, int out_bytes)
+UmmaPlan wide_shape(int batch, int n, int cin, int cout, int out_bytes)
 {
     const int nz = PAIR ? n / 2 : n;
     const long long tiles = static_cast<long long>(batch) * (n / kX) * (n / (PAIR ? 8 : 16)) * nz;
     const int sms = sm_count();
-    WideShape sh;
+    UmmaPlan sh;
     consider<64, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
     consider<64, 1, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
     consider<32, 4, PAIR>(sh, tiles, nz, cin, cout, out_bytes, sms);
@@ -653,7 +647,7 @@ WideShape wide_shape(int batch, int n, int cin, int cout, int out_bytes)
 }
 
 template <int CO, int R, bool PAIR, typename TO>
-cudaError_t launch_wide(const WideShape &sh, long long tiles, const __nv_bfloat16 *x, const __nv_bfloat16 *w,
+cudaError_t launch_wide(const UmmaPlan &sh, long long tiles, const __nv_bfloat16 *x, const __nv_bfloat16 *w,
                         const float *bias, TO *y, int n, int cin, int cout, int act, int *err, cudaStream_t s,
                         bool chained)
 {
@@ -666,11 +660,10 @@ cudaError_t launch_wide(const WideShape &sh, long long tiles, const __nv_bfloat1
 }
 
 template <bool PAIR, typename TO>
-cudaError_t run_wide(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
+cudaError_t run_wide(const UmmaPlan &sh, const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
                      int cin, int cout, int act, int *err, cudaStream_t s, bool chained)
 {
     const long long tiles = static_cast<long long>(batch) * (n / kX) * (n / (PAIR ? 8 : 16)) * (PAIR ? n / 2 : n);
-    const WideShape sh = wide_shape<PAIR>(batch, n, cin, cout, static_cast<int>(sizeof(TO)));
     auto go = [&](auto co, auto r) {
         return launch_wide<decltype(co)::value, decltype(r)::value, PAIR, TO>(sh, tiles, x, w, bias, y, n, cin, cout, act,
                                                                               err, s, chained);
@@ -706,9 +699,11 @@ int tensor_core_errors(bool reset)
 // with FP32 output 24^3 x 8, 16 -> 16 18.6 us here and 12.8 there, 40^3 x 3, 16
 // -> 16 25.0 and 20.6, but 24^3 x 8, 128 -> 128 224 and 375.  The mma.sync
 // kernel's time is within 5 % of the fit below; the tcgen05 one is taken where
-// it is estimated 10 % faster (of 353 layers, three are then slower than on
-// mma.sync by more than 2 %).
-bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout, int out_bytes)
+// it is estimated 4 % and (beyond the shortest) 1.5 us faster.  Of 353 layers
+// none is then slower than on mma.sync by more than 2 %, and 13 would be
+// faster here by 3 % or more.
+bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout, int out_bytes,
+                       UmmaPlan *plan)
 {
     static const bool on = std::getenv("DMRT_NN_NO_TCGEN05") == nullptr;
     const unsigned long long bases = reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(w) |
@@ -717,35 +712,41 @@ bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, i
     if (!(on && (bases & 15ull) == 0 && (cin == 8 || cin % 16 == 0) && cout % 16 == 0 && n % 8 == 0 &&
           vox * cin < (1LL << 31) && vox * batch / 128 < (1LL << 31) && cout / 16 < 65536))
         return false;
-    if (n % kY == 0) return true;
+    if (n % kY == 0) {
+        const bool narrow = cin <= 32 && (cout == 16 || cout == 32);
+        if (!narrow) *plan = wide_shape<false>(batch, n, cin, cout, out_bytes);
+        return true;
+    }
+    *plan = wide_shape<true>(batch, n, cin, cout, out_bytes);
     const double chunks = (cin + 15) / 16;
     const long long sms = sm_count(), blocks = vox * batch / 256 * (cout / 16);  // mma.sync blocks of 16 channels
     const double mma_sync = mma_sync_takes_32(vox * batch / 256, cout)
                                 ? 4.4 + chunks * (2.1 + 3.9 * static_cast<double>((blocks / 2 + sms - 1) / sms))
                                 : 3.6 + chunks * (2.3 + 2.64 * static_cast<double>((blocks + sms - 1) / sms));
-    return 1.1 * wide_shape<true>(batch, n, cin, cout, out_bytes).us <= mma_sync;
+    return 1.04 * plan->us + (mma_sync > 11.0 ? 1.5 : 0.0) <= mma_sync;
 }
 
 template <typename TO>
-cudaError_t conv3d_umma(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
-                        int cin, int cout, int act, cudaStream_t s, bool chained)
+cudaError_t conv3d_umma(const UmmaPlan &plan, const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y,
+                        int batch, int n, int cin, int cout, int act, cudaStream_t s, bool chained)
 {
     int *err = umma_error_word();
     if (!err) return cudaErrorInvalidValue;
-    if (n % kY == 0 && cin <= 32 && (cout == 16 || cout == 32)) {
+    if (plan.co == 0) {
         if (cout == 16 && cin <= 16) return launch_narrow<16, 2, TO>(x, w, bias, y, batch, n, cin, act, err, s, chained);
         if (cout == 16) return launch_narrow<16, 4, TO>(x, w, bias, y, batch, n, cin, act, err, s, chained);
         if (cin <= 16) return launch_narrow<32, 2, TO>(x, w, bias, y, batch, n, cin, act, err, s, chained);
         return launch_narrow<32, 4, TO>(x, w, bias, y, batch, n, cin, act, err, s, chained);
     }
-    if (n % kY == 0) return run_wide<false, TO>(x, w, bias, y, batch, n, cin, cout, act, err, s, chained);
-    return run_wide<true, TO>(x, w, bias, y, batch, n, cin, cout, act, err, s, chained);
+    if (n % kY == 0) return run_wide<false, TO>(plan, x, w, bias, y, batch, n, cin, cout, act, err, s, chained);
+    return run_wide<true, TO>(plan, x, w, bias, y, batch, n, cin, cout, act, err, s, chained);
 }
 
-template cudaError_t conv3d_umma<float>(const __nv_bfloat16 *, const __nv_bfloat16 *, const float *, float *, int, int,
-                                        int, int, int, cudaStream_t, bool);
-template cudaError_t conv3d_umma<__nv_bfloat16>(const __nv_bfloat16 *, const __nv_bfloat16 *, const float *,
-                                                __nv_bfloat16 *, int, int, int, int, int, cudaStream_t, bool);
+template cudaError_t conv3d_umma<float>(const UmmaPlan &, const __nv_bfloat16 *, const __nv_bfloat16 *, const float *,
+                                        float *, int, int, int, int, int, cudaStream_t, bool);
+template cudaError_t conv3d_umma<__nv_bfloat16>(const UmmaPlan &, const __nv_bfloat16 *, const __nv_bfloat16 *,
+                                                const float *, __nv_bfloat16 *, int, int, int, int, int, cudaStream_t,
+                                                bool);
 
 }  // namespace nn
 }  // namespace lbm

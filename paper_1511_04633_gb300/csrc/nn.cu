@@ -1480,8 +1480,9 @@ cudaError_t conv3d(const TI *x, const TW *w, const float *bias, TO *y, int batch
         // channel count and both base pointers must keep 16-byte alignment
         const bool aligned =
             ((reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(w)) & 15ull) == 0;
-        if (k == 3 && conv3d_umma_takes(x, w, y, batch, n, cin, cout, static_cast<int>(sizeof(TO))))
-            return conv3d_umma(x, w, bias, y, batch, n, cin, cout, act, s, chained);
+        UmmaPlan plan;
+        if (k == 3 && conv3d_umma_takes(x, w, y, batch, n, cin, cout, static_cast<int>(sizeof(TO)), &plan))
+            return conv3d_umma(plan, x, w, bias, y, batch, n, cin, cout, act, s, chained);
         if (k == 3 && aligned && (cin == 8 || cin % 16 == 0) && cout % 16 == 0 && n % kWtX == 0 &&
             n % kWtZ == 0) {
             const unsigned vtiles = static_cast<unsigned>(batch) * (n / kWtX) * (n / kWtY) * (n / kWtZ);

@@ -56,11 +56,16 @@ bool mma_sync_takes_32(long long voxel_tiles, int cout);
 // The 3^3 convolutions of bfloat16 x and w on the tcgen05 tensor cores
 // (conv_umma.cu): taken where the channel counts are multiples of 16 (cin
 // also 8), n a multiple of 8 and the three arrays 16-byte aligned, if they
-// are the faster ones.
-bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout, int out_bytes);
+// are the faster ones; *plan then says how.
+struct UmmaPlan {
+    int co = 0, R = 1, stages = 1;  // the wide kernel's tile; co = 0: the narrow kernel
+    double us = 0.0;                // estimated time
+};
+bool conv3d_umma_takes(const void *x, const void *w, const void *y, int batch, int n, int cin, int cout, int out_bytes,
+                       UmmaPlan *plan);
 template <typename TO>
-cudaError_t conv3d_umma(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y, int batch, int n,
-                        int cin, int cout, int act, cudaStream_t s, bool chained);
+cudaError_t conv3d_umma(const UmmaPlan &plan, const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias, TO *y,
+                        int batch, int n, int cin, int cout, int act, cudaStream_t s, bool chained);
 
 // dw (FP32, [tap][cout][cin]) of conv3d; scratch holds the per-chunk partials.
 template <typename TI>
