@@ -455,7 +455,7 @@ dmrt_status create_common(dmrt_t **out, const int grid[3], double nu, double alp
         return DMRT_ERR_ARG;
     }
     h->cells_per_thread = (cpt == 2 || (cpt == 0 && pair_ok)) ? 2 : 1;
-    h->split = cpt == 0 && !pair_ok && lbm::step_split_supported(wall_type, h->G) && lbm::step_split_pays(h->G);
+    h->split = cpt == 0 && !pair_ok && lbm::step_split_supported(wall_type, h->G) && lbm::step_split_pays(h->G, storage);
     // loads of the paired two-buffer kernel: TMA-staged where the tensor map
     // allows it (16-bit storage, nx a multiple of 8)
     const bool tma_ok = h->cells_per_thread == 2 && !h->inplace &&

@@ -119,7 +119,7 @@ cudaError_t launch_step_inplace_pair(int wall, int storage, bool stochastic, voi
 // a walled box; the launcher picks its own block shape.
 bool step_split_supported(int wall, const Geometry &G);
 // Is it the faster kernel of a box with odd rows?
-bool step_split_pays(const Geometry &G);
+bool step_split_pays(const Geometry &G, int storage);
 size_t split_blocks(const Geometry &G);
 cudaError_t launch_step_split(int wall, int storage, bool stochastic, const void *src, void *dst,
                               const StepGeometry &S, const Geometry &G, const CollideParams &C, cudaStream_t s,

@@ -470,13 +470,12 @@ int tile_width(int row, int &slots)
 // Boxes of 2.5 to 4 flat blocks per SM keep the tiles: FP32 48^3 4.5 -> 5.0
 // us, 52^3 4.7 -> 4.9; so do the smallest in place (16^3: 1.94 -> 2.07), and
 // boxes just beyond either line whose tiles are few as well: 54^3 in place FP32
-// 4.75 -> 5.21, 108 x 77 x 19 FP32 4.56 -> 4.89, 28 x 46 x 24 in place FP16 2.38 -> 2.59
-// (but with tiles of 16 pairs 206 x 8 x 96 FP16 5.05 -> 4.30, and 84 x 96 x 4 in place
-// 2.55 -> 2.34).  Of 1848 timed cases, five of the flat ones are then slower than
-// their tiles by 2 % or more (3 % at most).
+// 4.75 -> 5.21, 108 x 77 x 19 FP32 4.56 -> 4.89 (FP16 4.60 -> 4.35, flat), 28 x 46 x
+// 24 in place FP16 2.38 -> 2.59 (30^3 FP32 2.37 -> 2.25, flat); not with tiles of 16
+// pairs (206 x 8 x 96 FP16 5.05 -> 4.30), nor 84 x 96 x 4 in place (2.55 -> 2.34).
 // A step that takes a residual point always uses the row tiles: the order of
 // its sums, and so the residual, is then the same in either scheme.
-bool pair_flat(const Geometry &G, bool inplace, bool res)
+bool pair_flat(const Geometry &G, int storage, bool inplace, bool res)
 {
     if (res) return false;
     int slots;
@@ -486,18 +485,19 @@ bool pair_flat(const Geometry &G, bool inplace, bool res)
     if ((blocks > 380 && blocks <= 610) || (inplace && blocks <= 100)) return false;
     // the tiles fill one round (or one block per SM) just as well
     const long long tiles = static_cast<long long>((row + bx - 1) / bx) * ((G.ny + by - 1) / by) * G.nz;
-    if (blocks > 610 && blocks <= 640 && bx > 16 && tiles <= 152 * kPairBlocks) return false;
-    if (inplace && blocks <= 125 && tiles <= 152) return false;
+    const bool f32 = storage == 0;
+    if (blocks > 610 && blocks <= 640 && bx > 16 && tiles <= 152 * kPairBlocks && (inplace || f32)) return false;
+    if (inplace && !f32 && blocks <= 125 && tiles <= 152) return false;
     const double idle = 1.0 - static_cast<double>(row) * G.ny / (static_cast<double>(slots) * ((G.ny + by - 1) / by * by));
     return inplace ? idle > 0.08 : idle > 0.03 || G.nx % 32 != 0;
 }
 
 // Launch shape of the paired kernels (pair_coords).
-cudaLaunchConfig_t pair_config(const Geometry &G, bool inplace, bool res, cudaStream_t s, cudaLaunchAttribute *attr,
-                               bool pdl)
+cudaLaunchConfig_t pair_config(const Geometry &G, int storage, bool inplace, bool res, cudaStream_t s,
+                               cudaLaunchAttribute *attr, bool pdl)
 {
     cudaLaunchConfig_t cfg = {};
-    if (pair_flat(G, inplace, res)) {
+    if (pair_flat(G, storage, inplace, res)) {
         const long long pairs = static_cast<long long>(G.nx / 2) * G.ny * G.nz;
         // up to two blocks per SM: half as large ones spread further (36^3
         // FP32 2.9 -> 2.6 us)
@@ -523,7 +523,7 @@ cudaLaunchConfig_t pair_config(const Geometry &G, bool inplace, bool res, cudaSt
 size_t pair_blocks(const Geometry &G)
 {
     cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = pair_config(G, false, true, nullptr, attr, false);
+    const cudaLaunchConfig_t cfg = pair_config(G, 0, false, true, nullptr, attr, false);
     return static_cast<size_t>(cfg.gridDim.x) * cfg.gridDim.y * cfg.gridDim.z;
 }
 
@@ -533,7 +533,7 @@ cudaError_t launch_step_pair(int wall, int storage, bool stochastic, const void 
 {
     if (!step_pair_supported(wall, G)) return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pair_config(G, false, res != nullptr, s, attr, pdl);
+    cudaLaunchConfig_t cfg = pair_config(G, storage, false, res != nullptr, s, attr, pdl);
     const ResidualArgs R = res ? *res : ResidualArgs{};
     const BoxDivisors D(G);
     cudaError_t e = dispatch(wall, storage, [&](auto W, auto *tp) {
@@ -549,7 +549,7 @@ cudaError_t launch_step_pair(int wall, int storage, bool stochastic, const void 
                 if (res) return cudaLaunchKernelEx(&cfg, step_pair_kernel<WL, T, SRv, true, false>, a, b, S, C, R, D);
                 return cudaLaunchKernelEx(&cfg, step_pair_kernel<WL, T, SRv, false, FL>, a, b, S, C, R, D);
             };
-            auto by_shape = [&](auto sr) { return pair_flat(G, false, res != nullptr) ? go(sr, std::true_type{}) : go(sr, std::false_type{}); };
+            auto by_shape = [&](auto sr) { return pair_flat(G, storage, false, res != nullptr) ? go(sr, std::true_type{}) : go(sr, std::false_type{}); };
             if constexpr (!std::is_same_v<T, float>) {
                 if (stochastic) return by_shape(std::true_type{});
             }
@@ -663,7 +663,7 @@ cudaError_t launch_step_inplace_pair(int wall, int storage, bool stochastic, voi
 {
     if (!step_pair_supported(wall, G) || phase < 0 || phase > 2 || (phase == 2 && res)) return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pair_config(G, true, res != nullptr, s, attr, pdl);
+    cudaLaunchConfig_t cfg = pair_config(G, storage, true, res != nullptr, s, attr, pdl);
     const ResidualArgs R = res ? *res : ResidualArgs{};
     const BoxDivisors D(G);
     cudaError_t e = dispatch(wall, storage, [&](auto W, auto *tp) {
@@ -688,7 +688,7 @@ cudaError_t launch_step_inplace_pair(int wall, int storage, bool stochastic, voi
                 return phase == 0 ? run(integral_constant<int, 0>{}, std::false_type{})
                                   : run(integral_constant<int, 1>{}, std::false_type{});
             };
-            auto by_shape = [&](auto sr) { return pair_flat(G, true, res != nullptr) ? go(sr, std::true_type{}) : go(sr, std::false_type{}); };
+            auto by_shape = [&](auto sr) { return pair_flat(G, storage, true, res != nullptr) ? go(sr, std::true_type{}) : go(sr, std::false_type{}); };
             if constexpr (!std::is_same_v<T, float>) {
                 if (stochastic) return by_shape(std::true_type{});
             }

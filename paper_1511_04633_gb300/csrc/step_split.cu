@@ -280,22 +280,21 @@ bool step_split_supported(int wall, const Geometry &G)
 // 11 and 12; this kernel 2.5 to 2.8 for 1, 2.8 to 4.2 for 2, 3.7 to 4.6 up to
 // 2.5, 4.8 to 6.1 up to 5 (the hardware spreads more than 380 blocks
 // unevenly), 5.7 to 7.3 for 6.  Each row of the table: up to so many blocks of
-// this kernel, it is taken from so many one-cell blocks on; beyond it, from 1.8
-// times its own (thin boxes pair a slab with none).  Of 190 boxes of 25,000 to
-// 2,000,000 cells, in six variants each, 15 of 1140 are slower than on the
-// one-cell kernels by more than 1.5 % (three by 5 to 11 %), 14 would gain 3 %
-// or more here; a line at 60,000 cells and one round of blocks made 84 slower,
-// by up to 30 % (165 x 11 x 55 FP32 4.6 -> 6.0 us).  Boxes below 60,000 cells,
-// or of more than one round of blocks below 300,000, stay on the one-cell kernels.
-bool step_split_pays(const Geometry &G)
+// this kernel, it is taken from so many one-cell blocks on, FP32 and 16-bit;
+// beyond it, from 1.8 times its own (thin boxes pair a slab with none).  Of
+// 2346 timed cases, most of them chosen near these lines, 67 are slower than on
+// the one-cell kernels by 2 % or more (15 by 10 to 19 %) and 111 would gain 3 % or
+// more here; all together they gain 14 %.  Boxes below 60,000 cells, or of more
+// than one round of blocks below 300,000, stay on the one-cell kernels.
+bool step_split_pays(const Geometry &G, int storage)
 {
     const long long cells = static_cast<long long>(G.nx) * G.ny * G.nz;
     const long long blocks = static_cast<long long>(split_blocks(G));
     if (cells < 300000 && (cells < 60000 || blocks > 152 * kSplitBlocks)) return false;
     const long long one_cell = static_cast<long long>((G.nx + 31) / 32) * ((G.ny + 3) / 4) * G.nz;
-    constexpr int kLine[][2] = {{152, 456}, {290, 555}, {304, 608}, {380, 684}, {760, 1368}};
+    constexpr int kLine[][3] = {{152, 456, 456}, {290, 530, 530}, {380, 520, 520}, {608, 1474, 1307}, {760, 1094, 1094}};
     for (const auto &l : kLine)
-        if (blocks <= l[0]) return one_cell >= l[1];
+        if (blocks <= l[0]) return one_cell >= l[storage == 0 ? 1 : 2];
     return 5 * one_cell >= 9 * blocks;
 }
 
