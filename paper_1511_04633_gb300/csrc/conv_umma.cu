@@ -23,14 +23,16 @@
 //
 // Measured on GB300, kernel time per layer, before (a kernel that staged,
 // multiplied and waited in turn; mma.sync at 8^3) and now:
-//   16^3 x 4, 64 -> 64     29.1 -> 14.8 us     16^3 x 1, 64 -> 64    27.6 -> 8.7 us
-//   8^3 x 4, 128 -> 128    44.4 -> 16.2 us     16^3 x 4, 32 -> 64    15.4 -> 11.6 us
-//   64^3 x 2, 64 -> 64      561 -> 168 us      64^3 x 1, 128 -> 128  1057 -> 266 us
-//   64^3 x 4, 16 -> 16     42.1 -> 37.7 us     32^3 x 4, 32 -> 32    20.9 -> 18.4 us
-//   56^3 x 8, 16 -> 64      317 -> 233 us      (mma.sync before)
-// (873 TFLOP/s at 64^3, 128 -> 128: 46 % of the measured bf16 rate.)  Every
-// output is bitwise that of the kernels before: the K = 16 slices are added
-// in the same order, and tcgen05 and mma.sync add a slice alike.
+//   16^3 x 4, 64 -> 64     29.1 -> 14.8 us     16^3 x 1, 64 -> 64    27.6 -> 8.9 us
+//   8^3 x 4, 128 -> 128    44.4 -> 16.6 us     16^3 x 4, 32 -> 64    15.4 -> 11.2 us
+//   64^3 x 2, 64 -> 64      561 -> 163 us      64^3 x 1, 128 -> 128  1057 -> 263 us
+//   64^3 x 4, 16 -> 16     42.1 -> 37.6 us     32^3 x 4, 32 -> 32    20.9 -> 17.5 us
+//   56^3 x 8, 16 -> 64      317 -> 232 us      (mma.sync before)
+// (880 TFLOP/s at 64^3, 128 -> 128: 47 % of the measured bf16 rate.)  The wide
+// kernel's outputs are bitwise those of the mma.sync kernel: the K = 16 slices
+// are added in the same order, and tcgen05 and mma.sync add a slice alike.  The
+// narrow one adds the slices of a tap one after another, which is the same
+// for up to 16 input channels.
 //
 // Each wait is bounded; one that runs out sets *err, and the CTA drains its
 // copies and MMAs before it releases its TMEM and exits.
@@ -79,7 +81,7 @@ __device__ __forceinline__ void store8(__nv_bfloat16 *p, const float *v)
 // Sixteen consecutive channels (p 16-byte aligned; wide: 32-byte aligned).  A
 // warp's lanes store to 32 different lines, and each store instruction visits
 // every line: 32-byte stores make half the visits of 16-byte ones (48^3 x 6,
-// 16 -> 32 channels, FP32 output: 47.4 -> 42.9 us).
+// 16 -> 32 channels, FP32 output: 47.4 -> 41.6 us).
 __device__ __forceinline__ void store32(void *p, const uint4 &a, const uint4 &b)
 {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
@@ -596,7 +598,7 @@ cudaError_t launch_narrow(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const 
     const int per_sm = std::min({KG == 2 ? 4 : 2, static_cast<int>(kSmemPerSm / (smem + 1024u)), 512 / (kAcc * CO)});
     // every resident CTA takes an equal share, of at least kMinRun planes (a
     // run loads two planes more than it computes; runs of at least 4 left SMs
-    // idle: 32^3, 32 -> 32 channels 12.4 -> 9.8 us)
+    // idle: 32^3, 32 -> 32 channels 14.5 -> 12.4 us back to back)
     const long long planes = static_cast<long long>(batch) * (n / kX) * (n / kY) * n;
     const long long ctas = std::min<long long>(std::max(1, per_sm) * sm_count(), (planes + kMinRun - 1) / kMinRun);
     return launch_chained(kernel, static_cast<unsigned>(ctas), kThreads, smem, s, chained, x, w, bias, y, n, cin, act,
